@@ -116,7 +116,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     pdl_launch_dependents();
     const int G = p.Hq / p.Hkv;
     const int PR = p.T * G;
-    const int qt = blockIdx.x, kvh = blockIdx.y;
+    // a chain's query tiles see more keys the later they are: the longest start first
+    const int qt = p.causal ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x, kvh = blockIdx.y;
     const int s = blockIdx.z / p.S, split = blockIdx.z % p.S;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -167,7 +168,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     // they may be read before the dependency wait.  Pages entirely below seq_len - block_B hold committed
     // context that no kernel of this pass writes, so the producer prefetches them before the wait as well.
     const int P = p.seq_len[s];
-    const int n_keys = P + p.T;
+    // keys any row of this tile sees: all of them, or, in a chain, those up to the tile's last node
+    const int n_keys = P + (p.causal ? (min((qt + 1) * QT, PR) - 1) / G + 1 : p.T);
     const int n_tiles = (n_keys + KT - 1) / KT;
     // ceil-distribution: the extra tiles go to the first splits, because the last split already carries the
     // costlier masked tiles and the partial page
@@ -373,7 +375,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
         asm volatile("cp.async.commit_group;" ::);
         // the row's ancestor words travel while the copies are in flight
         uint64_t anc0 = ~0ull, anc1 = ~0ull;               // no mask: every extra key is visible
-        if (p.anc) {
+        if (p.anc && !p.causal) {
             const uint64_t *a = p.anc + ((size_t)s * p.T + node) * p.W;
             anc0 = a[0];
             anc1 = p.W > 1 ? a[1] : 0ull;
@@ -421,7 +423,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
                 // without a mask).  b0 = index of the first key among the extra keys; negative inside the context.
                 const int b0 = key0 + cg * KPT - P;
                 uint32_t vis;
-                if (b0 >= 0) {
+                if (p.causal) {
+                    const int n_vis = node + 1 - b0;      // leading visible keys of this thread
+                    vis = n_vis >= 32 ? 0xffffffffu : n_vis <= 0 ? 0u : ((1u << n_vis) - 1u);
+                } else if (b0 >= 0) {
                     const uint64_t lo = b0 >= 64 ? anc1 : anc0, hi = b0 >= 64 ? 0ull : anc1;
                     const int sh = b0 & 63;
                     vis = (uint32_t)(sh == 0 ? lo : ((lo >> sh) | (hi << (64 - sh))));

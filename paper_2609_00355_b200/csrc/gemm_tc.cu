@@ -88,6 +88,7 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
     const int f0 = tile_idx * FT;
     const int split = blockIdx.y;
     const int r0 = (a.rows_fastest ? blockIdx.x : blockIdx.z) * 128;
+    const int xr0 = r0 + a.x_row0;                       // first row inside X
     const int ktiles = a.K / BK;
     const int kt0 = (int)((long long)split * ktiles / a.S), kt1 = (int)((long long)(split + 1) * ktiles / a.S);
     const int nk = kt1 - kt0;
@@ -147,8 +148,8 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
             {
                 if (i + 1 == a.stall_kstep1) continue;
                 unsigned char *xs = smem + (size_t)i * stage_bytes + BM * 128;
-                tma_load_2d(xs, &map_x, &bars.full[i], (kt0 + i) * BK, r0);
-                if (NB > NP) tma_load_2d(xs + NP * 128, &map_x, &bars.full[i], (kt0 + i) * BK, a.x_lo_row + r0);
+                tma_load_2d(xs, &map_x, &bars.full[i], (kt0 + i) * BK, xr0);
+                if (NB > NP) tma_load_2d(xs + NP * 128, &map_x, &bars.full[i], (kt0 + i) * BK, a.x_lo_row + xr0);
             }
             int issued = pre;
             for (int i = pre; i < nk; ++i) {
@@ -159,8 +160,8 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
                 unsigned char *slot = smem + (size_t)s * stage_bytes;
                 mbar_expect_tx(&bars.full[s], (uint32_t)stage_bytes);
                 load_w(i, slot, &bars.full[s]);
-                tma_load_2d(slot + BM * 128, &map_x, &bars.full[s], (kt0 + i) * BK, r0);
-                if (NB > NP) tma_load_2d(slot + BM * 128 + NP * 128, &map_x, &bars.full[s], (kt0 + i) * BK, a.x_lo_row + r0);
+                tma_load_2d(slot + BM * 128, &map_x, &bars.full[s], (kt0 + i) * BK, xr0);
+                if (NB > NP) tma_load_2d(slot + BM * 128 + NP * 128, &map_x, &bars.full[s], (kt0 + i) * BK, a.x_lo_row + xr0);
                 issued = i + 1;
             }
             if (*abort_flag) {
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
             float inv = 1.f;
             if (a.ssq && t < NP && r0 + t < a.R) {   // NP <= 128 < 256 epilogue threads
                 float ss = 0.f;
-                for (int i = 0; i < a.n_ssq; ++i) ss += __ldcg(a.ssq + (size_t)i * a.ssq_stride + r0 + t);
+                for (int i = 0; i < a.n_ssq; ++i) ss += __ldcg(a.ssq + (size_t)i * a.ssq_stride + xr0 + t);
                 inv = rsqrtf(ss / (float)a.K + a.eps);
             }
             if (t < 128) inv_rms[t] = inv;

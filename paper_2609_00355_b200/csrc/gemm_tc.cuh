@@ -10,6 +10,7 @@ constexpr int kTopkTileCap = 16;     // candidate keys a (tile, row) pair may em
 
 struct TcGemmArgs {
     int Nout, K, R, S;          // W [Nout][K], X [R][K]; S = split-K factor (modes 0, 3, 4; 1 otherwise)
+    int x_row0;                 // mode 2: the R rows start at this row of X (and of the row statistics); results are 0-based
     int x_lo_row;               // > 0: X is two-term (hi + lo, both bf16); the lo plane starts at this row of the X map
     // mode 0: fp32 planes Y[split][r][f]; mode 2: optional fp32 logits Y[r][f] (may be nullptr)
     float *Y;

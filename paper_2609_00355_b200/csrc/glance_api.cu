@@ -50,6 +50,11 @@ int choose_split(int Nout, int K, int rows, bool two_term) {
     return s;
 }
 
+// Rows of one prefill pass (bounded by the sequence's capacity).  Every pass reads all weights, so a pass of N rows
+// costs their 14 GB at the 7B widths whatever N is, until the tensor work of the rows is as long (about 300 rows with
+// two-term activations).  At 2048 rows the weights are 10 % of the pass and the activations take 0.3 GB of workspace.
+constexpr int kPrefillRows = 2048;
+
 struct Workspace {
     float *x;            // [Rmax][H] residual stream
     bf16 *xn;            // [2][Rmax][H] bf16(x * gain) as two terms (hi plane, lo plane); so are attn and act
@@ -62,9 +67,8 @@ struct Workspace {
     float *ssq;            // [n_ssq][Rmax] per-tile sums of squares of the residual rows
     float *rope_cos, *rope_sin;
     double *inv_freq;      // [d/2]
-    uint64_t *chain_anc;   // [N][W] prefill chain mask
-    bf16 *hidden_tmp;      // [head layers][N][H] prefill: tapped hidden states of the chunk
-    int32_t *argmax_tmp;   // [N]
+    bf16 *hidden_tmp;      // [head layers][Rchunk][H] prefill: tapped hidden states of the chunk
+    int32_t *argmax_tmp;   // [1]
     int32_t *status;
     unsigned long long *am_keys;   // [Rlog] packed arg-max keys, zero between launches
     int32_t *am_counter;
@@ -78,18 +82,18 @@ struct Workspace {
 };
 
 struct Dims {
-    int Rmax, Rlog, qkv_out, qd, W, n_ssq;
+    int Rmax, Rlog, Rchunk, qkv_out, qd, n_ssq;
 };
 
 Dims make_dims(const glance_config &c) {
     Dims d;
     d.Rmax = c.max_batch * std::max(c.tree_N, 2 * c.block_B);
-    d.Rmax = std::max(d.Rmax, c.tree_N);
+    d.Rchunk = (int)std::min<long long>(kPrefillRows, (long long)c.max_pages_per_seq * kPage);
+    d.Rmax = std::max(d.Rmax, d.Rchunk);
     d.Rlog = c.max_batch * std::max(c.tree_N, c.block_B);
     d.qkv_out = (c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim;
     d.qd = c.n_q_heads * c.head_dim;
     d.n_ssq = (c.hidden + 127) / 128;
-    d.W = (c.tree_N + 63) / 64;
     return d;
 }
 
@@ -116,9 +120,8 @@ Workspace carve(const glance_config &c, const Dims &d, unsigned char *base) {
     w.rope_cos = (float *)take(R * (c.head_dim / 2) * 4);
     w.rope_sin = (float *)take(R * (c.head_dim / 2) * 4);
     w.inv_freq = (double *)take((size_t)(c.head_dim / 2) * 8);
-    w.chain_anc = (uint64_t *)take((size_t)c.tree_N * d.W * 8);
-    w.hidden_tmp = (bf16 *)take((size_t)(c.head_layers > 1 ? c.head_layers : 1) * c.tree_N * H * 2);
-    w.argmax_tmp = (int32_t *)take((size_t)c.tree_N * 4);
+    w.hidden_tmp = (bf16 *)take((size_t)(c.head_layers > 1 ? c.head_layers : 1) * d.Rchunk * H * 2);
+    w.argmax_tmp = (int32_t *)take(4);
     w.status = (int32_t *)take(256);
     w.am_keys = (unsigned long long *)take((size_t)d.Rlog * 8);
     w.am_counter = (int32_t *)take(256);
@@ -283,6 +286,7 @@ struct PassInfo {
     int Rq;                // rows that continue after the K/V write (queries)
     int batch, T;          // attention: T query rows / extra keys per sequence
     const uint64_t *anc;   // or nullptr
+    bool causal;           // the rows of a sequence are a chain (prefill)
     const glance_seqs *seqs;
     int seq_off;           // first sequence (prefill of one sequence of a batch)
 };
@@ -343,13 +347,18 @@ void run_layer(glance_ctx *ctx, const LayerW &w, bf16 *pool_layer, const PassInf
         g.v_off = (size_t)c.n_kv_heads * kPage * c.head_dim; g.head_stride = (size_t)kPage * c.head_dim;
         g.rope_cos = ws.rope_cos; g.rope_sin = ws.rope_sin;
         g.Hq = c.n_q_heads; g.Hkv = c.n_kv_heads; g.head_dim = c.head_dim; g.Rq = ps.Rq;
-        gemm(ctx, 4, w.wqkv, ws.xn, xr, g);
+        const bf16 *wqkv = w.wqkv;
+        if (ps.Rq == 0) {     // no row continues as a query (prefill of the head's context): the K and V features only
+            wqkv += (size_t)d.qd * c.hidden;
+            g.Nout = d.qkv_out - d.qd; g.Hq = 0; g.S = choose_split(g.Nout, c.hidden, ps.R, false);
+        }
+        gemm(ctx, 4, wqkv, ws.xn, xr, g);
     }
     if (ps.Rq == 0) return;
     AttnParams ap;
     ap.batch = ps.batch; ap.T = ps.T; ap.Hq = c.n_q_heads; ap.Hkv = c.n_kv_heads; ap.d = c.head_dim;
     ap.q = ws.q; ap.q_lo = ws.q + (size_t)xr * d.qd; ap.pool_layer = pool_layer; ap.geom = geom; ap.page_table = page_table; ap.seq_len = seq_len;
-    ap.anc = ps.anc; ap.W = (ps.T + 63) / 64; ap.out = ws.attn; ap.out_lo = ws.attn + (size_t)xr * d.qd;
+    ap.anc = ps.anc; ap.causal = ps.causal ? 1 : 0; ap.W = (ps.T + 63) / 64; ap.out = ws.attn; ap.out_lo = ws.attn + (size_t)xr * d.qd;
     ap.S = attention_tc_splits(ps.T, c.n_q_heads / c.n_kv_heads, c.n_kv_heads, ps.batch, c.head_dim);
     ap.status = ws.status;
     ap.lo_skip = ctx->attn_lo_skip; ap.lo_skip_min_keys = ctx->attn_lo_min_keys;
@@ -395,6 +404,7 @@ void run_target(glance_ctx *ctx, const PassInfo &ps, bf16 *hidden_out, float *lo
     if (argmax) {   // logits are stored only on request
         TcGemmArgs g{};
         g.Nout = c.vocab; g.K = c.hidden; g.R = ps.R; g.S = 1; g.Y = logits; g.ldy = c.vocab; g.argmax = argmax;
+        if (ps.causal) { g.x_row0 = ps.R - 1; g.R = 1; }     // a prefill decides one token, after its last row
         g.x_lo_row = 0;      // logits only decide an arg-max / top-k: one term is enough
         if (ctx->sample_on) {
             g.sample_pos = ctx->ws.row_pos; g.sample_seed = ctx->sample_seed; g.sample_inv_t = ctx->sample_inv_t;
@@ -534,31 +544,33 @@ int32_t glance_prefill(glance_ctx *ctx, const glance_seqs *seqs, int32_t seq, co
     const glance_config &c = ctx->cfg;
     Workspace &ws = ctx->ws;
     cudaStream_t st = ctx->stream;
-    const int N = c.tree_N;
-    for (int done = 0; done < count; done += N) {
-        const int n = std::min(N, count - done);
+    // equal chunks of at most Rchunk rows: a short last one would stream all weights for little work
+    const int chunks = (count + ctx->dims.Rchunk - 1) / ctx->dims.Rchunk;
+    for (int ch = 0; ch < chunks; ++ch) {
+        const int done = (int)((long long)count * ch / chunks), n = (int)((long long)count * (ch + 1) / chunks) - done;
         const bool last = (done + n == count);
         const KvGeom tg = geom_of(ctx, seqs);
         const int32_t *pt = seqs->page_table + (size_t)seq * c.max_pages_per_seq;
         VerifySetup vs{};
-        vs.batch = 1; vs.N = N; vs.d = c.head_dim; vs.theta = c.rope_theta;
+        vs.batch = 1; vs.N = n; vs.d = c.head_dim; vs.theta = c.rope_theta;
         vs.seq_len = seqs->seq_len + seq; vs.token = nullptr; vs.depth = nullptr;
         vs.row_embeds = embeds ? (const bf16 *)embeds + (size_t)done * c.hidden : nullptr;
         vs.row_ids = ids ? ids + done : nullptr;
-        vs.count = n; vs.chain_anc = ws.chain_anc; vs.embed = ctx->embed; vs.gain = ctx->ln1[0]; vs.vocab = c.vocab;
+        vs.group_rows = c.tree_N; vs.group_off = done % c.tree_N;
+        vs.embed = ctx->embed; vs.gain = ctx->ln1[0]; vs.vocab = c.vocab;
         vs.capacity = c.max_pages_per_seq * kPage; vs.geom = tg; vs.page_table = pt; vs.out = rowout_of(ctx);
         vs.meta = meta_of(ctx); vs.status = ws.status;
         LAUNCH(ctx, KIND_SETUP, launch_setup_verify(vs, st));
-        PassInfo ps{N, N, 1, N, ws.chain_anc, seqs, seq};
+        PassInfo ps{n, n, 1, n, nullptr, true, seqs, seq};
         run_target(ctx, ps, ws.hidden_tmp, nullptr, last ? ws.argmax_tmp : nullptr);
         // head context K/V of the new positions (Section 3.2: keys and values are the target's hidden states): every
         // head layer projects the hidden states of the target layer it taps with its own weights into its own pool
         for (int i = 0; i < head_depth(c); ++i) {
             const glance_head_layer &hl = ctx->head_layer[i];
             DraftSetup ds{};
-            ds.batch = 1; ds.B = c.block_B; ds.FR = N; ds.d = c.head_dim; ds.theta = c.rope_theta;
+            ds.batch = 1; ds.B = c.block_B; ds.FR = n; ds.d = c.head_dim; ds.theta = c.rope_theta;
             ds.seq_len = seqs->seq_len + seq; ds.root = seqs->root + seq;
-            ds.feat = ws.hidden_tmp + (size_t)i * N * c.hidden; ds.feat_count = nullptr;
+            ds.feat = ws.hidden_tmp + (size_t)i * n * c.hidden; ds.feat_count = nullptr;
             ds.count_const = n; ds.n_block = 0; ds.embed = ctx->embed; ds.mask_embed = (const bf16 *)ctx->head.mask_embed;
             ds.gain_block = (const bf16 *)hl.ln1; ds.gain_feat = (const bf16 *)hl.ctx_norm;
             ds.vocab = c.vocab; ds.capacity = c.max_pages_per_seq * kPage; ds.geom = tg; ds.page_table = pt;
@@ -566,7 +578,7 @@ int32_t glance_prefill(glance_ctx *ctx, const glance_seqs *seqs, int32_t seq, co
             LAUNCH(ctx, KIND_SETUP, launch_setup_draft(ds, st));
             LayerW hw{(const bf16 *)hl.ln2, (const bf16 *)hl.wqkv, (const bf16 *)hl.wo, (const bf16 *)hl.wgu,
                       (const bf16 *)hl.wd};
-            PassInfo hp{N, 0, 1, N, nullptr, seqs, seq};
+            PassInfo hp{n, 0, 1, n, nullptr, true, seqs, seq};
             run_layer(ctx, hw, (bf16 *)seqs->head_kv_pool + (size_t)i * tg.layer_stride(), hp, nullptr, nullptr);
         }
         LAUNCH(ctx, KIND_CONTROL, launch_prefill_advance(seqs->seq_len + seq, seqs->root + seq, seqs->feat_count + seq,
@@ -612,7 +624,7 @@ int32_t glance_draft_block(glance_ctx *ctx, const glance_seqs *seqs, int32_t *to
         ds.out = rowout_of(ctx); ds.meta = meta_of(ctx); ds.status = ws.status;
         LAUNCH(ctx, KIND_SETUP, launch_setup_draft(ds, st));
         LayerW hw{(const bf16 *)hl.ln2, (const bf16 *)hl.wqkv, (const bf16 *)hl.wo, (const bf16 *)hl.wgu, (const bf16 *)hl.wd};
-        PassInfo ps{R, R1, batch, B, nullptr, seqs, 0};
+        PassInfo ps{R, R1, batch, B, nullptr, false, seqs, 0};
         const bf16 *next_gain = i + 1 < HL ? (const bf16 *)ctx->head_layer[i + 1].ln1 : (const bf16 *)ctx->head.final_norm;
         run_layer(ctx, hw, (bf16 *)seqs->head_kv_pool + (size_t)i * hgeom.layer_stride(), ps, next_gain, nullptr);
     }
@@ -654,11 +666,11 @@ static int32_t verify_common(glance_ctx *ctx, const glance_seqs *seqs, const gla
     VerifySetup vs{};
     vs.batch = batch; vs.N = N; vs.d = c.head_dim; vs.theta = c.rope_theta;
     vs.seq_len = seqs->seq_len; vs.token = tree->token; vs.depth = tree->depth; vs.row_embeds = nullptr;
-    vs.row_ids = nullptr; vs.count = 0; vs.chain_anc = nullptr; vs.embed = ctx->embed; vs.gain = ctx->ln1[0];
+    vs.row_ids = nullptr; vs.embed = ctx->embed; vs.gain = ctx->ln1[0];
     vs.vocab = c.vocab; vs.capacity = c.max_pages_per_seq * kPage; vs.geom = geom_of(ctx, seqs);
     vs.page_table = seqs->page_table; vs.out = rowout_of(ctx); vs.meta = meta_of(ctx); vs.status = ws.status;
     LAUNCH(ctx, KIND_SETUP, launch_setup_verify(vs, ctx->stream));
-    PassInfo ps{batch * N, batch * N, batch, N, tree->anc, seqs, 0};
+    PassInfo ps{batch * N, batch * N, batch, N, tree->anc, false, seqs, 0};
     ctx->ent_on = true;
     run_target(ctx, ps, (bf16 *)hidden, logits_dbg, decisions);
     ctx->ent_on = false;
@@ -745,7 +757,7 @@ int32_t glance_debug_attention(glance_ctx *ctx, const glance_seqs *seqs, int32_t
     AttnParams ap;
     ap.batch = seqs->batch; ap.T = T; ap.Hq = c.n_q_heads; ap.Hkv = c.n_kv_heads; ap.d = c.head_dim;
     ap.q = (const bf16 *)q; ap.q_lo = (const bf16 *)q_lo; ap.pool_layer = (const bf16 *)seqs->kv_pool + (size_t)layer * geom.layer_stride();
-    ap.geom = geom; ap.page_table = seqs->page_table; ap.seq_len = seqs->seq_len; ap.anc = anc; ap.W = (T + 63) / 64;
+    ap.geom = geom; ap.page_table = seqs->page_table; ap.seq_len = seqs->seq_len; ap.anc = anc; ap.causal = 0; ap.W = (T + 63) / 64;
     ap.out = (bf16 *)out; ap.out_lo = (bf16 *)out_lo; ap.S = attention_tc_splits(T, c.n_q_heads / c.n_kv_heads, c.n_kv_heads, seqs->batch, c.head_dim);
     ap.status = ctx->ws.status;
     ap.lo_skip = ctx->attn_lo_skip; ap.lo_skip_min_keys = ctx->attn_lo_min_keys;

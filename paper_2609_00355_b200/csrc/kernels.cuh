@@ -26,8 +26,10 @@ struct VerifySetup {
     const int32_t *depth;       // [batch][N] (mode tree) or nullptr (chain: depth = i)
     const bf16 *row_embeds;     // prefill: [count][H] or nullptr
     const int32_t *row_ids;     // prefill: [count] or nullptr
-    int count;                  // prefill: valid rows
-    uint64_t *chain_anc;        // prefill: [N][W] written with the causal chain mask
+    // prefill (token == nullptr): N rows of one sequence, a causal chain.  The page budget is checked for groups of
+    // group_rows rows counted from the start of the call (this launch starts group_off rows into a group): a group
+    // whose first position + group_rows exceeds the capacity is reported and writes no K/V.
+    int group_rows, group_off;
     const bf16 *embed;          // [V][H]
     const bf16 *gain;           // first norm's gain
     int vocab;
@@ -45,7 +47,7 @@ struct DraftSetup {
     int batch, B, FR, d;
     float theta;
     const int32_t *seq_len, *root;
-    const bf16 *feat;           // [batch][FR][H]: FR = B (round) or tree_N (prefill head-context update)
+    const bf16 *feat;           // [batch][FR][H]: FR = B (round) or the chunk's rows (prefill head-context update)
     const int32_t *feat_count;  // [batch] or nullptr (then count_const rows, appended at seq_len)
     int count_const;
     int n_block;                // B (round) or 0 (prefill: only feature rows)
@@ -96,7 +98,7 @@ struct WalkCommit {
 };
 void launch_walk_commit(const WalkCommit &p, cudaStream_t st);
 
-// prefill bookkeeping: seq_len += count, root = argmax[count-1], feat_count = 0
+// prefill bookkeeping: seq_len += count, root = *argmax (if given), feat_count = 0
 void launch_prefill_advance(int32_t *seq_len, int32_t *root, int32_t *feat_count, const int32_t *argmax, int count,
                             cudaStream_t st);
 
@@ -110,6 +112,7 @@ struct AttnParams {
     const int32_t *page_table;
     const int32_t *seq_len;
     const uint64_t *anc;         // [batch][T][W] or nullptr (all T extra keys visible)
+    int causal;                  // 1: extra key j is visible to rows j.. (a chain of any length; anc is not read)
     int W;
     bf16 *out;                   // [batch*T][Hq*d]
     bf16 *out_lo;                // second term of the two-term output, or nullptr

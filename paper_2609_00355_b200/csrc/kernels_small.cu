@@ -93,8 +93,8 @@ __device__ __forceinline__ void emit_row(const RowOut &o, int r, const bf16 *src
 }
 
 // Verify-pass rows (Algorithm 1 line 3: pack the root and the tree).  Row r = s*N + i is node i of
-// sequence s at rotary position P + depth[i]; its K/V go to cache row P + i.  In prefill mode the rows are
-// a causal chain of `count` given embeddings / token ids and the chain's ancestor mask is emitted.
+// sequence s at rotary position P + depth[i]; its K/V go to cache row P + i.  In prefill mode the N rows are
+// a causal chain of given embeddings / token ids.
 __global__ void __launch_bounds__(128) setup_verify_kernel(VerifySetup p) {
     const int r = blockIdx.x;
     const int s = r / p.N, i = r % p.N;
@@ -103,8 +103,10 @@ __global__ void __launch_bounds__(128) setup_verify_kernel(VerifySetup p) {
     int depth = prefill ? i : p.depth[r];
     if (!prefill && (depth < 0 || depth > kMaxBlock)) depth = 0;
     if (threadIdx.x == 0) {
-        // a sequence without room for its N rows is reported once, as a capacity fault, and writes no K/V at all
-        const bool fits = P >= 0 && P + p.N <= p.capacity;
+        // rows without room for their whole group (a tree's N rows; group_rows of a prefill) are reported once, as a
+        // capacity fault, and write no K/V at all
+        const int first = prefill ? i - (p.group_off + i) % p.group_rows : 0;
+        const bool fits = P >= 0 && P + first + (prefill ? p.group_rows : p.N) <= p.capacity;
         if (!fits) set_status(p.status, GLANCE_E_CAPACITY);
         p.meta.seq[r] = s;
         p.meta.pos[r] = P + depth;
@@ -113,23 +115,11 @@ __global__ void __launch_bounds__(128) setup_verify_kernel(VerifySetup p) {
     fill_rope_row(p.meta, r, P + depth, p.d, p.theta);
     const bf16 *src = nullptr;
     if (prefill) {
-        if (i < p.count) {
-            if (p.row_embeds) src = p.row_embeds + (size_t)i * p.out.H;
-            else {
-                int t = p.row_ids[i];
-                if (t < 0 || t >= p.vocab) { t = 0; if (threadIdx.x == 0) set_status(p.status, GLANCE_E_BOUNDS); }
-                src = p.embed + (size_t)t * p.out.H;
-            }
-        }
-        // causal chain mask: row i sees rows 0..i
-        const int W = (p.N + 63) >> 6;
-        if (threadIdx.x < W) {
-            int w = threadIdx.x;
-            uint64_t bits;
-            if (i >= 64 * (w + 1) - 1) bits = ~0ull;
-            else if (i < 64 * w) bits = 0ull;
-            else bits = (~0ull) >> (63 - (i - 64 * w));
-            p.chain_anc[(size_t)i * W + w] = bits;
+        if (p.row_embeds) src = p.row_embeds + (size_t)i * p.out.H;
+        else {
+            int t = p.row_ids[i];
+            if (t < 0 || t >= p.vocab) { t = 0; if (threadIdx.x == 0) set_status(p.status, GLANCE_E_BOUNDS); }
+            src = p.embed + (size_t)t * p.out.H;
         }
     } else {
         int t = p.token[r];
@@ -553,7 +543,7 @@ __global__ void prefill_advance_kernel(int32_t *seq_len, int32_t *root, int32_t 
                                        int count) {
     if (threadIdx.x == 0) {
         seq_len[0] += count;
-        if (argmax) root[0] = argmax[count - 1];
+        if (argmax) root[0] = argmax[0];
         feat_count[0] = 0;
     }
 }

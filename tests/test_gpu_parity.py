@@ -427,6 +427,30 @@ def test_prefill_state_tiny(tiny_run):
     tiny_run.check_head_state()
 
 
+@pytest.mark.parametrize("n_img,n_txt", [(1, 16), (100, 29), (2040, 9), (2100, 2001)])
+def test_prefill_passes_of_many_rows(harness, n_img, n_txt):
+    """Prefill calls on both sides of a pass's 2048 rows and of the kernels' row tiles: state and cache against the oracle."""
+    run = harness.ParityRun(synth.CONFIGS["tiny"].replace(n_img=n_img, n_txt=n_txt))
+    run.check_state()
+    run.check_head_state()
+
+
+@pytest.mark.parametrize("first,count,status", [(0, 512, 0), (0, 513, -3), (3, 504, 0), (3, 505, -3)])
+def test_prefill_page_budget_by_groups_of_tree_rows(harness, first, count, status):
+    """Rows are admitted in groups of tree_N rows counted from the start of the call (512 positions, tree_N = 8)."""
+    cfg = synth.CONFIGS["tiny"]
+    eng = make_engine(cfg, max_len=512)
+    assert eng.pages_per_seq == 8 and cfg.tree_N == 8
+    eng.seq_len[0] = first
+    eng.glance_prefill(0, ids=torch.zeros(count, dtype=torch.int32, device="cuda"))
+    assert eng.glance_poll_status() == status
+    assert int(eng.seq_len[0]) == first + count
+    K, V = eng.gather_kv(0, 1, 512)
+    written = (K.abs().amax(dim=(1, 2)) > 0).nonzero().flatten().tolist()
+    whole = (512 - first) // 8 * 8                        # rows of the groups that fit
+    assert written == list(range(first, first + min(count, whole)))
+
+
 def test_rounds_tiny_drafted_trees(tiny_run):
     """Tiny config, trees from the library's own draft (random head: short accepts)."""
     for _ in range(4):
