@@ -19,8 +19,7 @@
 // drains and frees its TMEM before it returns.
 #include <cuda.h>
 
-#include "gemm_tc.cuh"
-#include "tc_ptx.cuh"
+#include "gemm_epilogue.cuh"
 
 namespace glance {
 
@@ -38,24 +37,6 @@ struct alignas(8) Barriers {
     uint32_t tmem_base;
     int abort_flag;
 };
-
-// Philox4x32-10 (Salmon et al., SC 2011): the counter-based generator behind the sampling mode's noise field.
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
-        c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
-        k.x += 0x9E3779B9u;
-        k.y += 0xBB67AE85u;
-    }
-    return c;
-}
-// standard Gumbel noise from one 32-bit word: u = ((w >> 9) + 0.5) 2^-23 lies strictly inside (0,1)
-__device__ __forceinline__ float gumbel_from_word(uint32_t w) {
-    const float u = ((float)(w >> 9) + 0.5f) * 1.1920928955078125e-07f;
-    return -logf(-logf(u));
-}
 
 // MODE 0: fp32 planes              MODE 1: SwiGLU (64 gate + 64 up rows per tile)   MODE 2: arg-max (+ optional logits)
 // MODE 3: split-K over a cluster, residual add + bf16 copy scaled by the next norm's gain + sum of squares
@@ -595,65 +576,7 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
     }
-    if (MODE == 2) {
-        // the last CTA to finish turns the merged keys into token ids and re-arms keys and counter
-        __shared__ int is_last;
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) is_last = (atomicAdd(a.counter, 1) == (int)(gridDim.x * gridDim.y * gridDim.z) - 1);
-        __syncthreads();
-        if (is_last) {
-            __threadfence();
-            for (int r = threadIdx.x; r < a.R; r += blockDim.x) {
-                const unsigned long long k = __ldcg(a.keys + r);
-                a.argmax[r] = unpack_id(k);
-                a.keys[r] = 0ull;
-            }
-            if (threadIdx.x == 0) *a.counter = 0;
-            if (a.ent_out) {
-                // entropy of every root row from the per-tile statistics: H = (M + log L) - T / L, merged in a fixed order
-                __shared__ float red_m[NTHR / 32], red_l[NTHR / 32], red_t[NTHR / 32];
-                const int tiles = (a.Nout + BM - 1) / BM;
-                const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31;
-                for (int sq = 0; sq < a.ent_batch && sq * a.ent_N < a.R; ++sq) {
-                    float M = -INFINITY, L = 0.f, T = 0.f;
-                    for (int tl = threadIdx.x; tl < tiles; tl += blockDim.x) {
-                        const float *src = a.ent_part + ((size_t)tl * a.ent_batch + sq) * 3;
-                        const float m = __ldcg(src), l = __ldcg(src + 1), t = __ldcg(src + 2);
-                        const float nm = fmaxf(M, m);
-                        const float c0 = (M == -INFINITY) ? 0.f : __expf(M - nm), c1 = __expf(m - nm);
-                        L = L * c0 + l * c1;
-                        T = T * c0 + t * c1;
-                        M = nm;
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const float m = __shfl_xor_sync(0xffffffffu, M, o), l = __shfl_xor_sync(0xffffffffu, L, o);
-                        const float t = __shfl_xor_sync(0xffffffffu, T, o);
-                        const float nm = fmaxf(M, m);
-                        const float c0 = (M == -INFINITY) ? 0.f : __expf(M - nm), c1 = (m == -INFINITY) ? 0.f : __expf(m - nm);
-                        L = L * c0 + l * c1;
-                        T = T * c0 + t * c1;
-                        M = nm;
-                    }
-                    if (ln == 0) { red_m[wid] = M; red_l[wid] = L; red_t[wid] = T; }
-                    __syncthreads();
-                    if (threadIdx.x == 0) {
-                        float gm = -INFINITY;
-                        for (int w = 0; w < NTHR / 32; ++w) gm = fmaxf(gm, red_m[w]);
-                        float gl = 0.f, gt = 0.f;
-                        for (int w = 0; w < NTHR / 32; ++w) {
-                            const float c = (red_m[w] == -INFINITY) ? 0.f : __expf(red_m[w] - gm);
-                            gl += red_l[w] * c;
-                            gt += red_t[w] * c;
-                        }
-                        a.ent_out[sq] = (gm + logf(gl)) - gt / gl;
-                    }
-                    __syncthreads();
-                }
-            }
-        }
-    }
+    if (MODE == 2) finish_argmax<NTHR>(a, (a.Nout + BM - 1) / BM);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -703,14 +626,24 @@ cudaError_t launch_mode(const TcGemmArgs &a, const CUtensorMap &mw, const CUtens
 }  // namespace
 
 bool tc_make_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows, uint32_t box_rows) {
+    const uint64_t dims[2] = {inner, rows}, steps[1] = {1};
+    const uint32_t box[2] = {BK, box_rows};
+    return tc_make_map_nd(map, base, 2, dims, steps, box);
+}
+
+bool tc_make_map_nd(CUtensorMap *map, const void *base, int n, const uint64_t *dims, const uint64_t *row_steps, const uint32_t *box) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    if (((uintptr_t)base & 15) != 0 || (inner * 2) % 16 != 0) return false;
-    cuuint64_t dims[2] = {inner, rows};
-    cuuint64_t strides[1] = {inner * 2};
-    cuuint32_t box[2] = {BK, box_rows};
-    cuuint32_t elem[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, elem,
+    if (((uintptr_t)base & 15) != 0 || (dims[0] * 2) % 16 != 0) return false;
+    cuuint64_t d[5], strides[4];
+    cuuint32_t b[5], elem[5];
+    for (int i = 0; i < n; ++i) {
+        d[i] = dims[i];
+        b[i] = box[i];
+        elem[i] = 1;
+        if (i > 0) strides[i - 1] = row_steps[i - 1] * dims[0] * 2;
+    }
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, n, const_cast<void *>(base), d, strides, b, elem,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }

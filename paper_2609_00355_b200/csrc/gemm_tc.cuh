@@ -29,8 +29,8 @@ struct TcGemmArgs {
     const int32_t *sample_pos;
     unsigned long long sample_seed;
     float sample_inv_t;
-    // mode 2, root-entropy log: rows r with r % ent_N == 0 are round roots; every tile leaves (max, sum exp, sum exp *
-    // logit) of its 128 features in ent_part [tiles][ent_batch][3] and the last CTA writes the entropy (nats) of
+    // mode 2, root-entropy log: rows r with r % ent_N == 0 are round roots; every part of the vocabulary (128 features of
+    // a tile, or 32 in gemm_wide_kernel) leaves its (max, sum exp, sum exp * logit) in ent_part [parts][ent_batch][3] and the last CTA writes the entropy (nats) of
     // sequence r / ent_N to ent_out; ent_out == nullptr: off
     float *ent_part, *ent_out;
     int ent_N, ent_batch;
@@ -66,18 +66,44 @@ struct TcGemmArgs {
     // runs out
     unsigned long long wait_limit_ns;
     int stall_kstep1;
-    // filled by launch_gemm_tc
+    int hook;                    // 1: a glance_debug_gemm launch (always on gemm_tc_kernel)
+    // gemm_wide_kernel: fp32 partial tiles of the items that several CTA pairs share, and their arrival counters
+    // [kWideCut][2] (zero between launches)
+    float *wide_planes;
+    int32_t *wide_counters;
+    int wide_pairs, wide_row_tiles, wide_rounds, wide_cut, wide_cutters;      // filled by launch_gemm_wide
+    // filled by launch_gemm_tc / launch_gemm_wide
     int np, stages, rows_fastest;
     uint32_t tmem_cols;
 };
 
 // 2-D bf16 tensor map {inner = K, rows}, box {64, box_rows}, 128-byte swizzle.  Host call, no device work.
 bool tc_make_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows, uint32_t box_rows);
+// the same with n <= 5 dimensions: dims[0] = inner, dimension i > 0 advances row_steps[i - 1] rows of `inner` elements
+bool tc_make_map_nd(CUtensorMap *map, const void *base, int n, const uint64_t *dims, const uint64_t *row_steps, const uint32_t *box);
 // activation rows per CTA, padded to the UMMA N granularity (box_rows of the X map)
 int tc_row_pad(int R);
 // mode: 0 fp32 planes, 1 SwiGLU, 2 arg-max, 3 cluster split-K + residual, 4 cluster split-K + rotary/KV write,
 // 5 per-tile top-k candidates + log-sum-exp shares.
 // map_w box_rows must be 128 (64 in mode 1), map_x box_rows tc_row_pad(R).
 cudaError_t launch_gemm_tc(int mode, TcGemmArgs a, const CUtensorMap &map_w, const CUtensorMap &map_x, cudaStream_t st);
+
+
+// ---- more than 128 rows (gemm_wide.cu) ---------------------------------------------------------------------------
+constexpr int kWideRows = 256;       // activation rows of a CTA pair's tile
+constexpr int kWidePairs = 74;       // one CTA per SM
+constexpr int kWideCut = kWidePairs;        // items that may be shared between pairs
+constexpr int kWideSmem = 198 * 1024;       // operand ring; the epilogue's static arrays take up to 28.5 KB beside it
+constexpr size_t kWidePlaneFloats = (size_t)kWidePairs * 2 * 2 * kWideRows * 128;   // two partial tiles per pair, two CTAs
+struct WideShape {
+    int row_tiles, np, items, pairs, rounds, cut, cutters;
+    long long steps;                 // 64-wide k-steps of the whole launch
+};
+WideShape wide_shape(int mode, int Nout, int K, int R);
+// map of W [Nout][K] for a mode of gemm_wide_kernel; the X map's box_rows is WideShape::np / 2
+bool wide_make_map(CUtensorMap *map, int mode, const void *W, int Nout, int K, int head_dim);
+// mode 1, 2, 3 or 4; S and the fields "filled by launch" are ignored
+cudaError_t launch_gemm_wide(int mode, TcGemmArgs a, const WideShape &s, const CUtensorMap &map_w, const CUtensorMap &map_x,
+                             cudaStream_t st);
 
 }  // namespace glance

@@ -55,6 +55,18 @@ int choose_split(int Nout, int K, int rows, bool two_term) {
 // two-term activations).  At 2048 rows the weights are 10 % of the pass and the activations take 0.3 GB of workspace.
 constexpr int kPrefillRows = 2048;
 
+// Whether a GEMM over more than 128 rows runs on CTA pairs with 256 x 256 tiles (gemm_wide.cu) or on the 128 x 128-row
+// tiles of gemm_tc_kernel.  It does where every pair has at least one whole item, or where the k-steps of a pair's share
+// outweigh the exchange of partial tiles.  Measured (us, 128 x 128 tiles -> pairs): gate/up 144 / 512 / 1536 rows 102 ->
+// 70, 203 -> 158, 606 -> 480; down 105 -> 53, 178 -> 115 (56 and 112 steps a pair); LM head at 512 rows 582 -> 450; but QKV
+// and O at 512 rows 27 -> 39 and 34 -> 46 (27 and 21 steps), the small model's gate/up at 708 rows 20 -> 31 (14 steps) and, with whole items
+// of only 16 steps each, at 2000 rows 54 -> 57.
+bool use_wide(int mode, int Nout, int K, int R) {
+    if (R <= 128 || mode < 1 || mode > 4) return false;
+    const WideShape s = wide_shape(mode, Nout, K, R);
+    return s.rounds > 0 ? s.pairs == kWidePairs && K >= 2048 : s.steps >= 48 * kWidePairs;
+}
+
 struct Workspace {
     float *x;            // [Rmax][H] residual stream
     bf16 *xn;            // [2][Rmax][H] bf16(x * gain) as two terms (hi plane, lo plane); so are attn and act
@@ -78,6 +90,8 @@ struct Workspace {
     float *tk_ml;                  // [vocab tiles][batch*B][2] (max, sum exp)
     int32_t *tk_cnt;               // [vocab tiles][batch*B] candidate keys emitted
     unsigned long long *tk_cand;   // [vocab tiles][batch*B][kTopkTileCap]
+    float *wide_planes;            // partial tiles of gemm_wide_kernel (only where its rule can choose it)
+    int32_t *wide_counters;        // [kWideCut][2], zero between launches
     size_t total;
 };
 
@@ -125,12 +139,17 @@ Workspace carve(const glance_config &c, const Dims &d, unsigned char *base) {
     w.status = (int32_t *)take(256);
     w.am_keys = (unsigned long long *)take((size_t)d.Rlog * 8);
     w.am_counter = (int32_t *)take(256);
-    w.ent_part = (float *)take((size_t)((c.vocab + 127) / 128) * c.max_batch * 3 * 4);
+    w.ent_part = (float *)take((size_t)((c.vocab + 127) / 128) * 4 * c.max_batch * 3 * 4);
     const size_t trows = (size_t)((c.vocab + 127) / 128) * c.max_batch * c.block_B;
     w.tk_thr = (uint32_t *)take((size_t)c.max_batch * c.block_B * kTopkTileCap * 4);
     w.tk_ml = (float *)take(trows * 2 * 4);
     w.tk_cnt = (int32_t *)take(trows * 4);
     w.tk_cand = (unsigned long long *)take(trows * kTopkTileCap * 8);
+    const bool wide = use_wide(4, d.qkv_out, c.hidden, d.Rmax) || use_wide(3, c.hidden, d.qd, d.Rmax) ||
+                      use_wide(1, 2 * c.ffn, c.hidden, d.Rmax) || use_wide(3, c.hidden, c.ffn, d.Rmax) ||
+                      use_wide(2, c.vocab, c.hidden, d.Rlog);
+    w.wide_planes = (float *)take(wide ? kWidePlaneFloats * 4 : 0);
+    w.wide_counters = (int32_t *)take((size_t)kWideCut * 2 * 4);
     w.total = off;
     return w;
 }
@@ -222,12 +241,14 @@ inline void prof_end(glance_ctx *ctx, bool prof, int kind, double bytes) {
         prof_end(ctx, prof_, kind, 0.0);         \
     } while (0)
 
+// box_rows < 0: the map of a weight matrix for mode -box_rows of gemm_wide_kernel
 const CUtensorMap *get_map(glance_ctx *ctx, const void *base, int inner, int rows, int box_rows) {
     auto key = std::make_tuple(base, inner, rows, box_rows);
     auto it = ctx->maps.find(key);
     if (it != ctx->maps.end()) return &it->second;
     CUtensorMap m;
-    if (!tc_make_map(&m, base, (uint64_t)inner, (uint64_t)rows, (uint32_t)box_rows)) {
+    if (!(box_rows < 0 ? wide_make_map(&m, -box_rows, base, rows, inner, ctx->cfg.head_dim)
+                       : tc_make_map(&m, base, (uint64_t)inner, (uint64_t)rows, (uint32_t)box_rows))) {
         ctx->map_error = true;
         return nullptr;
     }
@@ -237,8 +258,10 @@ const CUtensorMap *get_map(glance_ctx *ctx, const void *base, int inner, int row
 // Launches the weight-streaming GEMM described by `a` (mode: see gemm_tc.cuh) on X [R][K] (x_rows rows are
 // allocated behind X) and W [Nout][K], and tallies its algorithmic bytes.
 void gemm(glance_ctx *ctx, int mode, const bf16 *W, const bf16 *X, int x_rows, TcGemmArgs a) {
-    const CUtensorMap *mw = get_map(ctx, W, a.K, a.Nout, mode == 1 ? 64 : 128);
-    const CUtensorMap *mx = get_map(ctx, X, a.K, a.x_lo_row > 0 ? 2 * x_rows : x_rows, tc_row_pad(a.R));
+    const bool wide = a.hook == 0 && use_wide(mode, a.Nout, a.K, a.R);
+    const WideShape ws = wide ? wide_shape(mode, a.Nout, a.K, a.R) : WideShape{};
+    const CUtensorMap *mw = get_map(ctx, W, a.K, a.Nout, wide ? -mode : mode == 1 ? 64 : 128);
+    const CUtensorMap *mx = get_map(ctx, X, a.K, a.x_lo_row > 0 ? 2 * x_rows : x_rows, wide ? ws.np / 2 : tc_row_pad(a.R));
     if (!mw || !mx) return;
     a.keys = ctx->ws.am_keys; a.counter = ctx->ws.am_counter; a.status = ctx->ws.status;
     if (ctx->trace && ctx->trace_slots > 0) {
@@ -246,7 +269,9 @@ void gemm(glance_ctx *ctx, int mode, const bf16 *W, const bf16 *X, int x_rows, T
         ctx->trace_next++;
     }
     const bool prof = prof_begin(ctx);
-    if (launch_gemm_tc(mode, a, *mw, *mx, ctx->stream) != cudaSuccess) ctx->map_error = true;
+    a.wide_planes = ctx->ws.wide_planes; a.wide_counters = ctx->ws.wide_counters;
+    if ((wide ? launch_gemm_wide(mode, a, ws, *mw, *mx, ctx->stream) : launch_gemm_tc(mode, a, *mw, *mx, ctx->stream)) != cudaSuccess)
+        ctx->map_error = true;
     // weights once, activations in (both planes when two-term), results out
     double bytes = 2.0 * a.Nout * a.K + (a.x_lo_row > 0 ? 4.0 : 2.0) * a.R * a.K;
     if (mode == 0) bytes += 4.0 * a.S * a.R * a.Nout;
@@ -520,6 +545,7 @@ int32_t glance_create(const glance_config *cfg, const glance_target_weights *t, 
         cudaMemsetAsync(ws.status, 0, 256, ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ws.am_keys, 0, (size_t)d.Rlog * 8, ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ws.am_counter, 0, 256, ctx->stream) != cudaSuccess ||
+        cudaMemsetAsync(ws.wide_counters, 0, (size_t)kWideCut * 2 * 4, ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ws.tk_thr, 0, (size_t)cfg->max_batch * cfg->block_B * kTopkTileCap * 4, ctx->stream) != cudaSuccess) {
         delete ctx;
         return GLANCE_E_CUDA;
@@ -773,7 +799,7 @@ int32_t glance_debug_gemm(glance_ctx *ctx, int32_t mode, const void *W, const vo
     TcGemmArgs g{};
     g.Nout = Nout; g.K = K; g.R = R; g.S = mode == 0 ? S : 1; g.Y = Y; g.ldy = Nout; g.split_stride = (size_t)R * Nout;
     g.act = (bf16 *)act; g.F = Nout / 2; g.argmax = argmax;
-    g.stall_kstep1 = ctx->stall_kstep1; g.wait_limit_ns = ctx->stall_limit_ns;
+    g.hook = 1; g.stall_kstep1 = ctx->stall_kstep1; g.wait_limit_ns = ctx->stall_limit_ns;
     ctx->stall_kstep1 = 0; ctx->stall_limit_ns = 0;      // one shot
     gemm(ctx, mode, (const bf16 *)W, (const bf16 *)X, R, g);
     // the hook's operands are transient: their two descriptors are dropped again, everybody else's stay

@@ -451,6 +451,60 @@ def test_prefill_page_budget_by_groups_of_tree_rows(harness, first, count, statu
     assert written == list(range(first, first + min(count, whole)))
 
 
+@pytest.mark.parametrize("d,ffn,vocab,batch,N", [(64, 2112, 2500, 18, 123), (128, 2112, 2500, 18, 123), (128, 9536, 19000, 3, 43)])
+def test_batched_pass_equals_single_passes(harness, d, ffn, vocab, batch, N):
+    """A verify pass over many rows (CTA-pair GEMMs: whole and cut items, partial last tiles in both directions, one and
+    several row tiles) against the same sequences one by one (128-row GEMMs).  Operands are rounded alike; sums are added
+    in another order, which moves a result by at most a bf16 rounding here and there: within the 2e-2 of the other tests."""
+    base = synth.CONFIGS["tiny"].replace(n_layers=2, hidden=2112, n_q_heads=2304 // d, n_kv_heads=256 // d, head_dim=d, ffn=ffn,
+                                         vocab=vocab, tree_N=N, block_B=4, topk=2)
+    from paper_2609_00355_b200.binding import Engine
+    tw, hw = synth.make_weights(base, "cuda")
+    g = torch.Generator(device="cuda").manual_seed(5)
+    lens = [int(v) for v in np.random.default_rng(1).integers(3, 150, size=batch)]
+    tok = torch.randint(0, vocab, (batch, N), generator=g, device="cuda", dtype=torch.int32)
+    rng = np.random.default_rng(2)
+    trees = [synth.random_tree(N, 8, vocab, rng) for _ in range(batch)]
+    anc = np.zeros((batch, N, (N + 63) // 64), dtype=np.uint64)
+    for s, (_, parent, _) in enumerate(trees):
+        for i in range(N):
+            if i:
+                anc[s, i] = anc[s, parent[i]]
+            anc[s, i, i >> 6] |= np.uint64(1) << np.uint64(i & 63)
+
+    def run(seqs):
+        eng = Engine(base, tw, hw, batch=len(seqs), max_len=320)
+        pool = torch.Generator(device="cuda")
+        for j, s in enumerate(seqs):
+            pool.manual_seed(100 + s)
+            rows = torch.randn(2, 5, 2, base.n_kv_heads, 64, d, generator=pool, device="cuda").to(torch.bfloat16)
+            eng.kv_pool[:, eng.page_table[j, :5].long()] = rows
+            eng.seq_len[j] = lens[s]
+            eng.tree.token[j] = tok[s]
+            eng.tree.depth[j] = torch.from_numpy(trees[s][2]).cuda()
+            eng.tree.anc[j] = torch.from_numpy(anc[s].view(np.int64)).cuda()
+        ent = torch.zeros(len(seqs), device="cuda")
+        eng.glance_log_root_entropy(ent)
+        logits = torch.zeros(len(seqs), N, vocab, device="cuda")
+        eng.glance_verify_tree(logits_dbg=logits)
+        am = eng.argmax.clone()
+        assert torch.equal(am.long(), logits.argmax(-1))
+        eng.glance_verify_tree_sample(77, 1.0)
+        eng.check_device_status()
+        kv = [torch.stack(eng.gather_kv(j, 1, lens[s] + N)).float() for j, s in enumerate(seqs)]
+        return logits, eng.hidden_all[0].float(), kv, ent, eng.argmax.clone()
+
+    many = run(list(range(batch)))
+    same = 0
+    for s in range(batch):
+        one = run([s])
+        for x, y in ((many[0][s], one[0][0]), (many[1][s], one[1][0]), (many[2][s], one[2][0])):
+            assert float((x - y).abs().max()) <= 2e-2 * float(y.abs().max())
+        assert abs(float(many[3][s] - one[3][0])) <= 1e-3
+        same += int((many[4][s] == one[4][0]).sum())
+    assert same >= 0.95 * batch * N                       # draws differ at near-ties only
+
+
 def test_rounds_tiny_drafted_trees(tiny_run):
     """Tiny config, trees from the library's own draft (random head: short accepts)."""
     for _ in range(4):
