@@ -107,11 +107,17 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
         if (lane == 0) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(&map_w) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
+            // A layer's weights pass through L2 once and should not push out the activations, K/V rows and tables that the
+            // next kernels read (plain decoding 2981 -> 2955 us a token, a small model's round 441 -> 437; the LM heads,
+            // after which nothing of the pass is read, were 1 % slower with it)
+            const uint64_t w_policy = l2_evict_first();
             auto load_w = [&](int i, unsigned char *slot, uint64_t *bar) {
                 const int k0 = (kt0 + i) * BK;
                 if (MODE == 1) {
-                    tma_load_2d(slot, &map_w, bar, k0, f0);                       // gate rows
-                    tma_load_2d(slot + 64 * 128, &map_w, bar, k0, a.F + f0);     // up rows
+                    tma_load_2d(slot, &map_w, bar, k0, f0, w_policy);                       // gate rows
+                    tma_load_2d(slot + 64 * 128, &map_w, bar, k0, a.F + f0, w_policy);     // up rows
+                } else if (MODE == 3 || MODE == 4) {
+                    tma_load_2d(slot, &map_w, bar, k0, f0, w_policy);
                 } else {
                     tma_load_2d(slot, &map_w, bar, k0, f0);
                 }
@@ -133,9 +139,10 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
                 if (NB > NP) tma_load_2d(xs + NP * 128, &map_x, &bars.full[i], (kt0 + i) * BK, a.x_lo_row + xr0);
             }
             int issued = pre;
-            for (int i = pre; i < nk; ++i) {
-                const int s = i % stages;
-                const uint32_t ph = (uint32_t)(i / stages) & 1u;
+            // ring position and phase are carried along: a division per k-step lengthens the one thread's serial chain
+            int s = pre == stages ? 0 : pre;
+            uint32_t ph = pre == stages ? 1u : 0u;
+            for (int i = pre; i < nk; ++i, ph ^= (++s == stages) ? 1u : 0u, s = s == stages ? 0 : s) {
                 if (!mbar_wait(&bars.empty[s], ph ^ 1u, abort_flag, a.status, wait_limit)) break;
                 if (i + 1 == a.stall_kstep1) continue;        // test hook (nothing issued: `issued` keeps its value)
                 unsigned char *slot = smem + (size_t)s * stage_bytes;
@@ -160,9 +167,9 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
         if (lane == 0) {
             const uint32_t idesc = umma_idesc(NB);
             bool mok = true;
-            for (int i = 0; i < nk && mok; ++i) {
-                const int s = i % stages;
-                const uint32_t ph = (uint32_t)(i / stages) & 1u;
+            int s = 0;
+            uint32_t ph = 0;
+            for (int i = 0; i < nk && mok; ++i, ph ^= (++s == stages) ? 1u : 0u, s = s == stages ? 0 : s) {
                 if (!mbar_wait(&bars.full[s], ph, abort_flag, a.status, wait_limit)) { mok = false; break; }
                 if (trace && i == 0) trace[3] = global_ns();
                 tc_fence_after();
