@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(128) topk_stage1_kernel(const float *logits, i
     m = warp_max(m);
     float sum = 0.f;
 #pragma unroll
-    for (int i = 0; i < 32; ++i) sum += expf(val[i] - m);        // entries beyond V are -inf: they add exactly 0
+    for (int i = 0; i < 32; ++i) sum += expf(val[i] - (m == -INFINITY ? 0.f : m));   // -inf (and entries beyond V) add exactly 0
     sum = warp_sum(sum);
     if (lane == 0) {
         ml[((size_t)row * n_warps + gw) * 2] = m;

@@ -73,3 +73,37 @@ def test_topk_static_matches_draft_block_and_oracle_twice():
     rc = lib.glance_topk_static(big.data_ptr(), 65536, 2, 8, 1, ids.data_ptr(), lp.data_ptr(), None)
     assert rc == -3
     assert lib.glance_topk_static(None, 1, 2, 8, 1, ids.data_ptr(), lp.data_ptr(), None) == -1
+
+
+@pytest.mark.parametrize("V,k,kind", [(2, 1, "random"), (16, 16, "random"), (1000, 7, "ties"), (1025, 16, "random"), (33000, 16, "ties"),
+                                      (262144, 16, "random"), (262145, 3, "random"), (600000, 16, "random"), (600000, 16, "stripes"),
+                                      (70000, 5, "inf")])
+def test_topk_static_edges_of_spans_and_lists(V, k, kind):
+    """One span, its remainders, more spans than threads, many equal values, -inf entries, and keys concentrated in a few
+    spans, against the exact (logit desc, id asc) order on the CPU."""
+    from paper_2609_00355_b200 import binding
+    rng = np.random.default_rng(V + k)
+    x = rng.standard_normal((1, 3, V)).astype(np.float32)
+    if kind == "ties":
+        x = np.round(x * 2) / 2
+    elif kind == "stripes":                               # the best keys all in spans that one thread of the merge shares
+        x[..., : V // 1024 * 1024].reshape(1, 3, -1, 1024)[:, :, 0::256] += 20
+    elif kind == "inf":
+        x[..., 10:] = -np.inf
+    g = torch.from_numpy(x).cuda()
+    ids = torch.full((1, 2, k), -1, dtype=torch.int32, device="cuda")
+    lp = torch.full((1, 2, k), float("nan"), dtype=torch.float32, device="cuda")
+    for _ in range(2):
+        assert binding.glance_topk_static(g, k, ids, lp) == 0
+    torch.cuda.synchronize()
+    for j in range(2):
+        row = x[0, j + 1].astype(np.float64)
+        order = np.lexsort((np.arange(V), -row))[:k]
+        assert ids[0, j].cpu().tolist() == order.tolist()
+        m = row.max()
+        ref = row[order] - (m + np.log(np.exp(row - m).sum()))
+        got = lp[0, j].cpu().numpy()
+        fin = np.isfinite(ref)
+        assert np.array_equal(np.isfinite(got), fin)
+        # fp32 sums of V terms in blocks of 32 and more: 1e-6 of the log-sum-exp's scale
+        assert np.abs(got[fin] - ref[fin]).max() <= 4e-6 * max(1.0, float(np.abs(row[np.isfinite(row)]).max()) + np.log(V))
