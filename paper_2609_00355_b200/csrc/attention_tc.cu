@@ -363,13 +363,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
 #pragma unroll
             for (int k = 0; k < QT / RSTEP; ++k) {
                 const int r = tsm / CH + k * RSTEP;
+                // rows beyond the last query are zeros, not read: with one query a head, 121 of the tile's 128 rows would
+                // otherwise fetch the same two lines (plain decoding 2951 -> 2917 us a token)
                 int prr = qt * QT + r;
+                const uint32_t take = prr < PR ? 16u : 0u;
                 if (prr >= PR) prr = PR - 1;
                 const size_t off = ((size_t)(s * p.T + prr / G) * p.Hq + kvh * G + prr % G) * D + c * 8;
                 const uint32_t dst = dst0 + (uint32_t)(r * 128 + (((c & 7) ^ (r & 7)) << 4));
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(p.q + off));
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(p.q + off), "r"(take));
                 if (p.q_lo)
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)(SLABS * QT * 128)), "l"(p.q_lo + off));
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + (uint32_t)(SLABS * QT * 128)), "l"(p.q_lo + off), "r"(take));
             }
         }
         asm volatile("cp.async.commit_group;" ::);
