@@ -40,7 +40,7 @@ constexpr int NTHR = 64 + 32 * NEPI;
 constexpr int CSTEP = NEPI / 4 * 16;         // columns that the warps of a lane quarter cover together
 constexpr int PAIR = 2 * BM;                 // weight rows of a pair's tile
 constexpr int MAX_STAGES = 8;
-constexpr int FLIGHT = 3;                    // parts of a cut item in flight
+constexpr int FLIGHT = 4;                    // parts of a cut item in flight (3: down at 512 rows 113.5 instead of 110 us)
 constexpr size_t PLANE = (size_t)kWideRows * BM;   // floats of one CTA's partial tile
 
 struct alignas(8) WideBars {
@@ -334,15 +334,12 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
                     float4 *pl = plane_of(my_part);
                     for (int c = c0; c < NP; c += CSTEP) {
                         uint32_t v[16];
-                        if (ok) {
-                            tmem_ld16(acc + (uint32_t)c, v);
-                            tmem_ld_wait();
-                        }
+                        tmem_ld16(acc + (uint32_t)c, v);
+                        tmem_ld_wait();
 #pragma unroll
                         for (int j = 0; j < 16; j += 4)
                             if (c + j < rows)
-                                __stcg(pl + (size_t)((c + j) >> 2) * BM, ok ? make_float4(__uint_as_float(v[j]), __uint_as_float(v[j + 1]), __uint_as_float(v[j + 2]), __uint_as_float(v[j + 3]))
-                                                                           : make_float4(0.f, 0.f, 0.f, 0.f));
+                                __stcg(pl + (size_t)((c + j) >> 2) * BM, make_float4(__uint_as_float(v[j]), __uint_as_float(v[j + 1]), __uint_as_float(v[j + 2]), __uint_as_float(v[j + 3])));
                     }
                     __threadfence();
                     epilogue_sync();
@@ -395,13 +392,12 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
                     }
                     float v[16];
                     auto take_own = [&](bool first) {
+                        // (after a wait that gave up the columns hold anything: the launch's results are undefined then)
                         uint32_t w[16];
-                        if (ok) {
-                            tmem_ld16(acc + (uint32_t)c, w);
-                            tmem_ld_wait();
-                        }
+                        tmem_ld16(acc + (uint32_t)c, w);
+                        tmem_ld_wait();
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] = (first ? 0.f : v[j]) + (ok ? __uint_as_float(w[j]) : 0.f);
+                        for (int j = 0; j < 16; ++j) v[j] = first ? __uint_as_float(w[j]) : v[j] + __uint_as_float(w[j]);
                     };
                     if (n_parts == 1) {
                         take_own(true);
