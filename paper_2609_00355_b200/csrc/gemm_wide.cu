@@ -549,7 +549,9 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
                                 }
                             l += __shfl_xor_sync(0xffffffffu, l, 1);
                             tt += __shfl_xor_sync(0xffffffffu, tt, 1);
-                            if (in && (lane & 1) == 0 && row % a.ent_N == 0) {
+                            // the last pair tile's second half may lie wholly behind the vocabulary: it has no parts
+                            // (a part is kept for every 32 features of ceil(Nout / 128) tiles of 128)
+                            if (in && (lane & 1) == 0 && row % a.ent_N == 0 && (tile * 2 + (int)rank) * BM < a.Nout) {
                                 const int part = (tile * 2 + (int)rank) * 4 + q;
                                 float *dst = a.ent_part + ((size_t)part * a.ent_batch + row / a.ent_N) * 3;
                                 dst[0] = mx; dst[1] = l; dst[2] = tt;

@@ -84,7 +84,9 @@ struct Workspace {
     int32_t *status;
     unsigned long long *am_keys;   // [Rlog] packed arg-max keys, zero between launches
     int32_t *am_counter;
-    float *ent_part;       // [vocab tiles][max_batch][3] soft-max statistics of the root rows (entropy log)
+    // soft-max statistics of the root rows (entropy log): [parts][sequences of the pass][3], a part being 128 features
+    // (gemm_tc_kernel) or 32 (gemm_wide_kernel); sized for 32
+    float *ent_part;
     // draft top-k, fused into the LM head: per 128-feature tile and block row
     uint32_t *tk_thr;              // [batch*B][kTopkTileCap] running class maxima of every row (0 between launches)
     float *tk_ml;                  // [vocab tiles][batch*B][2] (max, sum exp)

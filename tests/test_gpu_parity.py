@@ -505,6 +505,41 @@ def test_batched_pass_equals_single_passes(harness, d, ffn, vocab, batch, N):
     assert same >= 0.95 * batch * N                       # draws differ at near-ties only
 
 
+@pytest.mark.parametrize("topk,vocab", [(1, 19000), (2, 19000), (8, 19000), (1, 18945), (1, 18944)])
+def test_draft_after_a_batched_pass_with_the_entropy_log(harness, topk, vocab):
+    """A vocabulary of an odd number of 128-feature tiles, more than 128 verify rows, every sequence slot in use: the
+    entropy statistics of the pass end where their buffer ends.  The draft's bounds lie behind it in the workspace, so the
+    next draft has to be the one of an engine that logs nothing, bit for bit; and the log agrees with the pass's logits."""
+    cfg = synth.CONFIGS["tiny"].replace(n_layers=1, hidden=2304, n_q_heads=16, n_kv_heads=2, head_dim=128, ffn=1024, vocab=vocab,
+                                        tree_N=48, block_B=8, topk=topk)
+    from paper_2609_00355_b200.binding import Engine
+    tw, hw = synth.make_weights(cfg, "cuda")
+    batch, drafts = 8, []
+    for log in (True, False):
+        eng = Engine(cfg, tw, hw, batch=batch, max_len=320)
+        pool = torch.Generator(device="cuda").manual_seed(7)
+        for t in (eng.kv_pool, eng.head_kv_all, eng.feat_all):
+            t.copy_(torch.randn(t.shape, generator=pool, device="cuda").to(torch.bfloat16))
+        eng.seq_len.copy_(torch.arange(100, 100 + batch, dtype=torch.int32))
+        eng.root.copy_(torch.arange(batch, dtype=torch.int32))
+        eng.feat_count.fill_(3)
+        eng.tree.token.copy_(torch.arange(batch * cfg.tree_N, dtype=torch.int32).reshape(batch, -1) % vocab)
+        eng.tree.anc.copy_(torch.ones(cfg.tree_N, dtype=torch.int64).view(1, -1, 1).expand_as(eng.tree.anc))
+        logits = torch.zeros(batch, cfg.tree_N, vocab, device="cuda")
+        if log:
+            ent = torch.full((batch,), float("nan"), device="cuda")
+            eng.glance_log_root_entropy(ent)
+        eng.glance_verify_tree(logits_dbg=logits)
+        if log:
+            lp = torch.log_softmax(logits[:, 0].double(), -1)
+            # fp32 exponentials and sums of V terms: 1e-6 of an entropy of about ten nats
+            assert float((ent.double() + (lp.exp() * lp).sum(-1)).abs().max()) <= 2e-5
+        eng.glance_draft_block()
+        eng.check_device_status()
+        drafts.append((eng.topk_ids.clone(), eng.topk_lp.clone()))
+    assert torch.equal(drafts[0][0], drafts[1][0]) and torch.equal(drafts[0][1], drafts[1][1])
+
+
 def test_rounds_tiny_drafted_trees(tiny_run):
     """Tiny config, trees from the library's own draft (random head: short accepts)."""
     for _ in range(4):
