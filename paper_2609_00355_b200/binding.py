@@ -19,7 +19,7 @@ EXPORTS = [
     "glance_seq_truncate", "glance_draft_block", "glance_build_tree", "glance_verify_tree",
     "glance_verify_tree_sample", "glance_log_root_entropy",
     "glance_accept_commit", "glance_commit_forced", "glance_poll_status", "glance_launch_count",
-    "glance_debug_attention", "glance_debug_gemm", "glance_profile_enable", "glance_profile_read",
+    "glance_debug_attention", "glance_debug_gemm", "glance_debug_gemm_wide", "glance_profile_enable", "glance_profile_read",
     "glance_topk_static", "glance_debug_trace", "glance_debug_attention_terms", "glance_debug_stall_next_gemm",
 ]
 
@@ -107,6 +107,9 @@ def load_library() -> C.CDLL:
     lib.glance_debug_gemm.restype = C.c_int32
     lib.glance_debug_gemm.argtypes = [C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
                                          C.c_int32, C.c_int32, C.c_int32, C.c_int32]
+    lib.glance_debug_gemm_wide.restype = C.c_int32
+    lib.glance_debug_gemm_wide.argtypes = [C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p,
+                                           C.c_void_p, C.c_void_p, C.c_int32, C.c_int32, C.c_int32]
     lib.glance_profile_enable.restype = C.c_int32
     lib.glance_profile_enable.argtypes = [C.c_void_p, C.c_int32]
     lib.glance_profile_read.restype = C.c_int32
@@ -321,6 +324,10 @@ class Engine:
     def glance_debug_gemm(self, mode: int, W, X, Y=None, act=None, argmax=None, S: int = 1):
         _check(self.lib.glance_debug_gemm(self.ctx, mode, _ptr(W), _ptr(X), _ptr(Y), _ptr(act), _ptr(argmax),
                                              W.shape[0], W.shape[1], X.shape[0], S), "glance_debug_gemm")
+
+    def glance_debug_gemm_wide(self, mode: int, W, X, terms: int = 1, Y=None, act=None, argmax=None, gain=None):
+        _check(self.lib.glance_debug_gemm_wide(self.ctx, mode, _ptr(W), _ptr(X), terms, _ptr(Y), _ptr(act), _ptr(argmax), _ptr(gain),
+                                               W.shape[0], W.shape[1], X.shape[0] // terms), "glance_debug_gemm_wide")
 
     def glance_debug_attention_terms(self, lo_skip: int, min_keys: int = 0):
         _check(self.lib.glance_debug_attention_terms(self.ctx, lo_skip, min_keys), "glance_debug_attention_terms")

@@ -66,7 +66,7 @@ struct TcGemmArgs {
     // runs out
     unsigned long long wait_limit_ns;
     int stall_kstep1;
-    int hook;                    // 1: a glance_debug_gemm launch (always on gemm_tc_kernel)
+    int hook;                    // 1: a glance_debug_gemm launch (gemm_tc_kernel), 2: glance_debug_gemm_wide (gemm_wide_kernel)
     // gemm_wide_kernel: fp32 partial tiles of the items that several CTA pairs share, and their arrival counters
     // [kWideCut][2] (zero between launches)
     float *wide_planes;

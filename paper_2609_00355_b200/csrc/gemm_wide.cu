@@ -22,7 +22,9 @@
 // under the main loop of the next.
 //
 // Warp roles: warp 0 = TMA producer, warp 1 = tensor memory + MMA issuer (first CTA of the pair), warps 2..9 = epilogue.
-// Every mbarrier wait is bounded; one that gives up records GLANCE_E_TIMEOUT.
+// Every mbarrier wait is bounded.  One that gives up records GLANCE_E_TIMEOUT and tells the other CTA of the pair: from the
+// item that it concerns on neither stores results, a cut item with a given-up part is finished by nobody (its counter still
+// returns to zero), and before the pair leaves it waits for the copies and MMAs that it has in flight.
 #include <cuda.h>
 
 #include <algorithm>
@@ -42,12 +44,15 @@ constexpr int PAIR = 2 * BM;                 // weight rows of a pair's tile
 constexpr int MAX_STAGES = 8;
 constexpr int FLIGHT = 4;                    // parts of a cut item in flight (3: down at 512 rows 113.5 instead of 110 us)
 constexpr size_t PLANE = (size_t)kWideRows * BM;   // floats of one CTA's partial tile
+constexpr int GIVEN_UP = 1 << 16;            // added to a cut item's arrival counter by a part that has no result
 
 struct alignas(8) WideBars {
     uint64_t full[MAX_STAGES], empty[MAX_STAGES];
     uint64_t acc_full[2], acc_empty[2];
+    uint64_t drained;
     uint32_t tmem_base;
     int abort_flag;
+    int issued;                              // k-steps that this CTA's producer has gone through
 };
 
 __device__ __forceinline__ void tma_load_pair(void *dst, const CUtensorMap *map, uint32_t bar_cluster, int c0, int c1, uint64_t policy) {
@@ -89,6 +94,32 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
 }
 __device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * NEPI) : "memory"); }
+// the same barrier, and whether every epilogue thread says yes
+__device__ __forceinline__ bool epilogue_all(bool yes) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "bar.red.and.pred q, 1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r) : "r"((uint32_t)yes), "n"(32 * NEPI) : "memory");
+    return r != 0;
+}
+// Bounded wait; giving up (or finding that another role did) also stops the other CTA of the pair.
+__device__ __forceinline__ bool pair_wait(WideBars &bars, uint64_t *bar, uint32_t parity, int32_t *status, uint64_t limit_ns) {
+    if (mbar_wait(bar, parity, &bars.abort_flag, status, limit_ns)) return true;
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(map_to_rank(smem_u32(&bars.abort_flag), cluster_rank() ^ 1u)), "r"(1) : "memory");
+    return false;
+}
+// takes bytes that no copy will deliver off a barrier's count
+__device__ __forceinline__ void mbar_complete_tx(uint64_t *bar, uint32_t bytes) {
+    asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bounded_wait(uint64_t *bar, uint32_t parity, uint64_t limit_ns) {
+    const uint64_t t0 = global_ns();
+    while (!mbar_try_wait(bar, parity))
+        if (global_ns() - t0 > limit_ns) break;
+}
 
 // The work of one pair, in order: its range [u0, u1) of the cut items' k-steps, then `rounds` whole items.
 struct Deal {
@@ -144,7 +175,7 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
     // consecutive features of a row with 16-byte accesses (2-byte stores, one per row and lane, took 1.3 us per chunk)
     constexpr int TS = 36;
     __shared__ __align__(16) float turn[NEPI][16 * TS];
-    __shared__ int sh_last;
+    __shared__ int sh_seen;                               // a cut item's counter: the others that are there
 
     const int NP = a.np, half_rows = NP / 2, stages = a.stages, terms = a.x_lo_row > 0 ? 2 : 1;
     const int x_bytes = half_rows * 128, stage_bytes = BM * 128 + terms * x_bytes;
@@ -152,6 +183,7 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
     const uint32_t rank = cluster_rank();
     const int FT = MODE == 1 ? BM : PAIR;                 // output features of a tile
     const Deal deal(a, blockIdx.x >> 1);
+    const uint64_t wait_limit = a.wait_limit_ns ? a.wait_limit_ns : kWaitLimitNs;
 
     // optional phase timestamps of the first CTA (test hook; a.trace is nullptr in normal use)
     unsigned long long *trace = (a.trace && blockIdx.x == 0) ? a.trace : nullptr;
@@ -167,7 +199,9 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
             mbar_init(&bars.acc_full[b], 1);
             mbar_init(&bars.acc_empty[b], 2 * NEPI);      // one arrival per epilogue warp of both CTAs
         }
+        mbar_init(&bars.drained, 1);
         bars.abort_flag = 0;
+        bars.issued = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -179,7 +213,6 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
     tc_fence_after();
     const uint32_t tmem_base = bars.tmem_base;
     const uint32_t acc_cols = a.tmem_cols / 2;            // columns between the two accumulators
-    volatile int *abort_flag = &bars.abort_flag;
     if (trace && threadIdx.x == 0) trace[1] = global_ns();
 
     if (warp == 0) {
@@ -205,6 +238,7 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
             int s = 0;                                    // ring slot of the next k-step, and the phase it waits for
             uint32_t phase = 1;
             bool waited = false, alive = true;
+            int n = 0;                                    // k-steps so far
             Segment sg;
             for (int i = 0; alive && segment(deal, i, sg); ++i) {
                 const int f = sg.item / a.wide_row_tiles * FT + (int)rank * (FT / 2);
@@ -215,32 +249,37 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
                     // weights depend on no kernel: they travel while the predecessor finishes
                     const int pre = min(sg.k1 - sg.k0, stages);
                     for (int j = 0; j < pre; ++j) {
+                        if (j + 1 == a.stall_kstep1) continue;        // test hook: this slot is never filled
                         if (rank == 0) mbar_expect_tx(&bars.full[j], (uint32_t)(2 * stage_bytes));
                         load_w(k + j, smem + (size_t)j * stage_bytes, full0 + 8 * j);
                     }
                     pdl_wait();
                     waited = true;
                     if (trace) trace[2] = global_ns();
-                    for (int j = 0; j < pre; ++j) load_x(k + j, smem + (size_t)j * stage_bytes, full0 + 8 * j);
+                    for (int j = 0; j < pre; ++j)
+                        if (j + 1 != a.stall_kstep1) load_x(k + j, smem + (size_t)j * stage_bytes, full0 + 8 * j);
                     k += pre;
+                    n = pre;
                     s = pre;
                     if (s == stages) { s = 0; phase = 0; }
                 }
                 for (; k < sg.k1; ++k) {
-                    if (!mbar_wait(&bars.empty[s], phase, abort_flag, a.status)) { alive = false; break; }
+                    if (!pair_wait(bars, &bars.empty[s], phase, a.status, wait_limit)) { alive = false; break; }
                     unsigned char *slot = smem + (size_t)s * stage_bytes;
-                    if (rank == 0) mbar_expect_tx(&bars.full[s], (uint32_t)(2 * stage_bytes));
-                    load_w(k, slot, full0 + 8 * s);
-                    load_x(k, slot, full0 + 8 * s);
+                    if (++n != a.stall_kstep1) {          // (test hook)
+                        if (rank == 0) mbar_expect_tx(&bars.full[s], (uint32_t)(2 * stage_bytes));
+                        load_w(k, slot, full0 + 8 * s);
+                        load_x(k, slot, full0 + 8 * s);
+                    }
                     if (++s == stages) { s = 0; phase ^= 1; }
                 }
             }
             if (!waited) pdl_wait();
-            if (*abort_flag) {
-                // copies in flight must land before the CTA may exit; the second CTA's are counted on the first CTA's
-                // barriers, so both allow them a fixed time that is far above any copy's
-                const uint64_t t0 = global_ns();
-                while (global_ns() - t0 < 1000000ull) __nanosleep(1000);
+            bars.issued = n;
+            // the last arrivals on this CTA's slots, which MMAs of the first CTA signal, come in before it may leave
+            for (int i = 0; alive && i < stages; ++i) {
+                alive = pair_wait(bars, &bars.empty[s], phase, a.status, wait_limit);
+                if (++s == stages) { s = 0; phase ^= 1; }
             }
         }
     } else if (warp == 1) {
@@ -253,11 +292,11 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
             Segment sg;
             for (int i = 0; ok && segment(deal, i, sg); ++i) {
                 const int b = i & 1;
-                if (!mbar_wait(&bars.acc_empty[b], ((uint32_t)(i >> 1) & 1u) ^ 1u, abort_flag, a.status)) break;
+                if (!pair_wait(bars, &bars.acc_empty[b], ((uint32_t)(i >> 1) & 1u) ^ 1u, a.status, wait_limit)) break;
                 tc_fence_after();
                 const uint32_t acc = tmem_base + (uint32_t)b * acc_cols;
                 for (int k = sg.k0; k < sg.k1; ++k) {
-                    if (!mbar_wait(&bars.full[s], phase, abort_flag, a.status)) { ok = false; break; }
+                    if (!pair_wait(bars, &bars.full[s], phase, a.status, wait_limit)) { ok = false; break; }
                     if (trace && first) trace[3] = global_ns();
                     first = false;
                     tc_fence_after();
@@ -282,6 +321,7 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
         const int c0 = ((warp - 2) >> 2) * 16;            // this warp's first column; its chunks are CSTEP columns apart
         const int t = threadIdx.x - 64;
         const uint32_t acc_empty0 = map_to_rank(smem_u32(&bars.acc_empty[0]), 0u);
+        bool alive = true;                                // no wait has given up so far (the same in every warp)
         Segment sg;
         for (int i = 0; segment(deal, i, sg); ++i) {
             const int b = i & 1;
@@ -319,20 +359,23 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
                 }
                 row_scale[b][t] = inv;
             }
-            bool ok = mbar_wait(&bars.acc_full[b], (uint32_t)(i >> 1) & 1u, abort_flag, a.status);
+            bool ok = alive && pair_wait(bars, &bars.acc_full[b], (uint32_t)(i >> 1) & 1u, a.status, wait_limit);
             ok = __all_sync(0xffffffffu, ok);
             tc_fence_after();
             const uint32_t acc = tmem_base + (uint32_t)b * acc_cols + ((uint32_t)(q * 32) << 16);
             if (trace && t == 0 && i == 0) trace[4] = global_ns();
-            bool finish = true;
+            int32_t *counter = a.wide_counters + sg.item * 2 + rank;
+            if (n_parts > 1 && t == 0) sh_seen = *reinterpret_cast<volatile int32_t *>(counter);
+            // One decision for the CTA; behind this barrier the row scales are there and part_f / part_k are free.  It holds
+            // for all later items too: a barrier that was given up in one phase may read as complete in the next.
+            alive = ok = epilogue_all(ok);
+            bool finish = ok;
             if (n_parts > 1) {
-                int32_t *counter = a.wide_counters + sg.item * 2 + rank;
-                if (t == 0) sh_last = *reinterpret_cast<volatile int32_t *>(counter) == n_parts - 1;   // all others are there
-                epilogue_sync();
-                finish = sh_last != 0;
+                int seen = sh_seen;
+                finish = (seen & (GIVEN_UP - 1)) == n_parts - 1;                // all others are there
                 if (!finish) {
                     float4 *pl = plane_of(my_part);
-                    for (int c = c0; c < NP; c += CSTEP) {
+                    for (int c = c0; ok && c < NP; c += CSTEP) {
                         uint32_t v[16];
                         tmem_ld16(acc + (uint32_t)c, v);
                         tmem_ld_wait();
@@ -343,19 +386,20 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
                     }
                     __threadfence();
                     epilogue_sync();
-                    if (t == 0) sh_last = atomicAdd(counter, 1) == n_parts - 1;
+                    if (t == 0) sh_seen = atomicAdd(counter, ok ? 1 : 1 + GIVEN_UP);
                     epilogue_sync();
-                    finish = sh_last != 0;
+                    seen = sh_seen;
+                    finish = (seen & (GIVEN_UP - 1)) == n_parts - 1;
                 }
                 if (finish) {
                     __threadfence();
                     if (t == 0) *counter = 0;             // ready for the next launch
+                    finish = ok && seen < GIVEN_UP;
                 }
-                epilogue_sync();                          // sh_last may be written again
+                epilogue_sync();                          // sh_seen may be written again
             }
             if (trace && t == 0 && i == 0) trace[7] = finish ? global_ns() : 0;
             if (finish) {
-                epilogue_sync();                          // row scales are there; part_f / part_k are free
                 float *tn = turn[warp - 2];
                 for (int c = c0; c < NP; c += CSTEP) {
                     const int n = min(16, rows - c);      // rows of this chunk (warp-uniform)
@@ -392,7 +436,6 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
                     }
                     float v[16];
                     auto take_own = [&](bool first) {
-                        // (after a wait that gave up the columns hold anything: the launch's results are undefined then)
                         uint32_t w[16];
                         tmem_ld16(acc + (uint32_t)c, w);
                         tmem_ld_wait();
@@ -609,6 +652,27 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
     }
     tc_fence_before();
     cluster_sync_all();                                   // neither CTA leaves while the other still uses its memory
+    if (*reinterpret_cast<volatile int *>(&bars.abort_flag)) {       // set in both CTAs or in neither
+        // MMAs in flight read both CTAs' shared memory and write both CTAs' tensor memory; copies in flight write shared
+        // memory and are counted on the first CTA's barriers
+        if (warp == 1 && lane == 0) {
+            if (rank == 0) umma_commit_pair(&bars.drained);
+            bounded_wait(&bars.drained, 0, wait_limit);
+        } else if (warp == 0 && lane == 0 && rank == 0) {
+            int theirs;
+            asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(theirs) : "r"(map_to_rank(smem_u32(&bars.issued), 1u)) : "memory");
+            const int mine = bars.issued, most = max(mine, theirs);
+            for (int j = max(0, most - stages); j < most; ++j) {
+                if (j + 1 == a.stall_kstep1) continue;    // issued by neither
+                if (j >= mine) mbar_expect_tx(&bars.full[j % stages], (uint32_t)stage_bytes);           // the peer's copies only
+                else if (j >= theirs) mbar_complete_tx(&bars.full[j % stages], (uint32_t)stage_bytes);  // without the peer's
+            }
+            for (int j = max(0, most - stages); j < most; ++j)
+                if (j + 1 != a.stall_kstep1) bounded_wait(&bars.full[j % stages], (uint32_t)(j / stages) & 1u, wait_limit);
+        }
+        __syncwarp();
+        cluster_sync_all();
+    }
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(a.tmem_cols) : "memory");

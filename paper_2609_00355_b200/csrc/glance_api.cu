@@ -92,7 +92,7 @@ struct Workspace {
     float *tk_ml;                  // [vocab tiles][batch*B][2] (max, sum exp)
     int32_t *tk_cnt;               // [vocab tiles][batch*B] candidate keys emitted
     unsigned long long *tk_cand;   // [vocab tiles][batch*B][kTopkTileCap]
-    float *wide_planes;            // partial tiles of gemm_wide_kernel (only where its rule can choose it)
+    float *wide_planes;            // partial tiles of gemm_wide_kernel, or nullptr where its rule never chooses it
     int32_t *wide_counters;        // [kWideCut][2], zero between launches
     size_t total;
 };
@@ -150,7 +150,7 @@ Workspace carve(const glance_config &c, const Dims &d, unsigned char *base) {
     const bool wide = use_wide(4, d.qkv_out, c.hidden, d.Rmax) || use_wide(3, c.hidden, d.qd, d.Rmax) ||
                       use_wide(1, 2 * c.ffn, c.hidden, d.Rmax) || use_wide(3, c.hidden, c.ffn, d.Rmax) ||
                       use_wide(2, c.vocab, c.hidden, d.Rlog);
-    w.wide_planes = (float *)take(wide ? kWidePlaneFloats * 4 : 0);
+    w.wide_planes = wide ? (float *)take(kWidePlaneFloats * 4) : nullptr;
     w.wide_counters = (int32_t *)take((size_t)kWideCut * 2 * 4);
     w.total = off;
     return w;
@@ -211,7 +211,7 @@ struct glance_ctx {
     int trace_slots = 0, trace_next = 0;
     // attention: which second bf16 terms the pure-context key tiles drop, and from which context length on
     int attn_lo_skip = 0, attn_lo_min_keys = 0;
-    // test hook, one shot: the next glance_debug_gemm launch withholds one ring slot and waits at most this long
+    // test hook, one shot: the next glance_debug_gemm(_wide) launch withholds one ring slot and waits at most this long
     int stall_kstep1 = 0;
     unsigned long long stall_limit_ns = 0;
 };
@@ -260,7 +260,7 @@ const CUtensorMap *get_map(glance_ctx *ctx, const void *base, int inner, int row
 // Launches the weight-streaming GEMM described by `a` (mode: see gemm_tc.cuh) on X [R][K] (x_rows rows are
 // allocated behind X) and W [Nout][K], and tallies its algorithmic bytes.
 void gemm(glance_ctx *ctx, int mode, const bf16 *W, const bf16 *X, int x_rows, TcGemmArgs a) {
-    const bool wide = a.hook == 0 && use_wide(mode, a.Nout, a.K, a.R);
+    const bool wide = a.hook == 0 ? use_wide(mode, a.Nout, a.K, a.R) : a.hook == 2;
     const WideShape ws = wide ? wide_shape(mode, a.Nout, a.K, a.R) : WideShape{};
     const CUtensorMap *mw = get_map(ctx, W, a.K, a.Nout, wide ? -mode : mode == 1 ? 64 : 128);
     const CUtensorMap *mx = get_map(ctx, X, a.K, a.x_lo_row > 0 ? 2 * x_rows : x_rows, wide ? ws.np / 2 : tc_row_pad(a.R));
@@ -807,6 +807,30 @@ int32_t glance_debug_gemm(glance_ctx *ctx, int32_t mode, const void *W, const vo
     // the hook's operands are transient: their two descriptors are dropped again, everybody else's stay
     ctx->maps.erase(std::make_tuple((const void *)W, K, Nout, mode == 1 ? 64 : 128));
     ctx->maps.erase(std::make_tuple((const void *)X, K, R, tc_row_pad(R)));
+    return finish(ctx);
+}
+
+int32_t glance_debug_gemm_wide(glance_ctx *ctx, int32_t mode, const void *W, const void *X, int32_t terms, float *Y, void *act,
+                               int32_t *argmax, const void *gain, int32_t Nout, int32_t K, int32_t R) {
+    if (!ctx || !W || !X || mode < 1 || mode > 3 || terms < 1 || terms > 2) return GLANCE_E_INVALID_ARG;
+    if (Nout < 1 || K < 64 || K % 64 || R <= 128 || R > std::min(ctx->dims.Rlog, ctx->dims.Rmax)) return GLANCE_E_INVALID_ARG;
+    if ((mode == 1 && (!act || Nout % 128)) || (mode == 2 && !argmax) ||
+        (mode == 3 && (!Y || !act || !gain || Nout % 64 || Nout > ctx->cfg.hidden)))
+        return GLANCE_E_INVALID_ARG;
+    if (!ctx->ws.wide_planes) return GLANCE_E_SHAPE;
+    TcGemmArgs g{};
+    g.Nout = Nout; g.K = K; g.R = R; g.S = 1; g.x_lo_row = terms == 2 ? R : 0; g.act = (bf16 *)act; g.F = Nout / 2; g.argmax = argmax;
+    if (mode == 3) {
+        g.x = Y; g.gain = (const bf16 *)gain; g.xb = (bf16 *)act; g.ssq_out = ctx->ws.ssq; g.ssq_stride = ctx->dims.Rmax;
+    } else {
+        g.Y = Y; g.ldy = Nout;
+    }
+    g.hook = 2; g.stall_kstep1 = ctx->stall_kstep1; g.wait_limit_ns = ctx->stall_limit_ns;
+    ctx->stall_kstep1 = 0; ctx->stall_limit_ns = 0;      // one shot
+    gemm(ctx, mode, (const bf16 *)W, (const bf16 *)X, R, g);
+    // (transient operands, as above)
+    ctx->maps.erase(std::make_tuple((const void *)W, K, Nout, -mode));
+    ctx->maps.erase(std::make_tuple((const void *)X, K, terms * R, wide_shape(mode, Nout, K, R).np / 2));
     return finish(ctx);
 }
 

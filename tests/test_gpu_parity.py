@@ -119,6 +119,100 @@ def test_gemm_tc_argmax(gemm_eng, V, K, R):
     assert torch.equal(am, am2)
 
 
+@pytest.fixture(scope="module")
+def wide_eng(harness):
+    return make_engine(synth.CONFIGS["tiny"].replace(n_layers=1, hidden=2304, ffn=8192, vocab=256, tree_N=128), batch=8, max_len=64)
+
+
+def _wide_operands(mode, Nout, K, R, terms):
+    g = torch.Generator(device="cuda").manual_seed(Nout + K + R + mode)
+    W = (torch.randn(Nout, K, generator=g, device="cuda") * 0.05).to(torch.bfloat16)
+    x = torch.randn(R, K, generator=g, device="cuda")
+    X = x.to(torch.bfloat16)
+    if terms == 2:
+        X = torch.cat([X, (x - X.float()).to(torch.bfloat16)])
+    ref = X.double().view(terms, R, K).sum(0) @ W.double().T
+    return g, W, X.contiguous(), ref
+
+
+# whole and cut items, an item of several parts, partial last tiles in both directions, one k-step, one and more row tiles
+@pytest.mark.parametrize("mode,Nout,K,R,terms", [
+    (1, 1408, 2304, 200, 2), (1, 20480, 256, 130, 2), (1, 128, 64, 129, 1), (1, 4096, 1024, 1000, 2),
+    (2, 19000, 320, 129, 1), (2, 1000, 2304, 600, 1), (2, 255, 64, 300, 1), (2, 18945, 1024, 256, 1),
+    (3, 2304, 8192, 144, 2), (3, 2112, 4096, 1024, 2), (3, 64, 64, 129, 1), (3, 192, 2304, 300, 2)])
+def test_gemm_wide(wide_eng, mode, Nout, K, R, terms):
+    """CTA-pair GEMM against a 64-bit matmul of the same bf16 terms: the bounds of the 128-row kernel's tests, sums in fp32
+    (1e-4 of the largest result), act one bf16 rounding of it (eight significant bits: half a unit in the last place is at
+    most 2^-8 of the value) and the same 1e-4 for the sums behind it."""
+    g, W, X, ref = _wide_operands(mode, Nout, K, R, terms)
+    bound = 1e-4 * float(ref.abs().max()) + 1e-5
+    runs = []
+    for rep in range(2):                                  # the second launch meets re-armed counters and keys
+        if mode == 1:
+            act = torch.full((R, Nout // 2), float("nan"), dtype=torch.bfloat16, device="cuda")
+            wide_eng.glance_debug_gemm_wide(1, W, X, terms, act=act)
+            want = torch.nn.functional.silu(ref[:, :Nout // 2]) * ref[:, Nout // 2:]
+            assert bool(((act.double() - want).abs() <= 2 ** -8 * want.abs() + 1e-4 * float(want.abs().max())).all())
+            runs.append((act,))
+        elif mode == 2:
+            am = torch.full((R,), -1, dtype=torch.int32, device="cuda")
+            Y = torch.full((R, Nout), float("nan"), device="cuda")
+            wide_eng.glance_debug_gemm_wide(2, W, X, terms, Y=Y, argmax=am)
+            assert float((Y.double() - ref).abs().max()) <= bound
+            assert np.array_equal(am.cpu().numpy(), O.argmax_lowest(Y.cpu()))
+            runs.append((Y, am))
+        else:
+            x0 = torch.randn(R, Nout, generator=torch.Generator(device="cuda").manual_seed(3), device="cuda")
+            gain = (torch.rand(Nout, generator=torch.Generator(device="cuda").manual_seed(4), device="cuda") + 0.5).to(torch.bfloat16)
+            Y, act = x0.clone(), torch.full((R, Nout), float("nan"), dtype=torch.bfloat16, device="cuda")
+            wide_eng.glance_debug_gemm_wide(3, W, X, terms, Y=Y, act=act, gain=gain)
+            assert float((Y.double() - (ref + x0.double())).abs().max()) <= bound
+            assert torch.equal(act, (Y * gain.float()).to(torch.bfloat16))
+            runs.append((Y, act))
+        assert wide_eng.glance_poll_status() == 0
+    assert all(torch.equal(a, b) for a, b in zip(*runs))  # parts are added in k order: run-to-run identical
+
+
+@pytest.mark.parametrize("mode,Nout,K,R,kstep,done", [
+    (3, 2304, 8192, 144, 2, []), (3, 2304, 8192, 144, 9, []),    # nine items, all cut: parts of 16 k-steps
+    # one cut item of four parts, then a whole one for each pair
+    (2, 19000, 1024, 256, 2, []), (2, 19000, 1024, 256, 9, [(0, 256)]),
+    # 160 items of four k-steps: 0..11, 12..85 and 86..159 are the first, second and third round of the twelve first pairs
+    (1, 40960, 256, 200, 1, []), (1, 40960, 256, 200, 5, [(0, 12 * 128), (24 * 128, 86 * 128)])])
+def test_bounded_wait_of_a_pair_runs_out(wide_eng, mode, Nout, K, R, kstep, done):
+    """As for the 128-row kernel, with CTA pairs: one ring slot of both CTAs is never filled, inside the first ring fill, in a
+    re-used slot, or in a pair's second item.  Every pair gives up, no tile from there on is written (items that were
+    complete before are), the host reads GLANCE_E_TIMEOUT, and the same launch again is correct."""
+    terms = 1 if mode == 2 else 2
+    g, W, X, ref = _wide_operands(mode, Nout, K, R, terms)
+    cols = Nout // 2 if mode == 1 else Nout
+    marker = -7.5
+    out = torch.full((R, cols), marker, device="cuda", dtype=torch.bfloat16 if mode == 1 else torch.float32)
+    act, am = torch.full((R, cols), marker, device="cuda", dtype=torch.bfloat16), torch.zeros(R, dtype=torch.int32, device="cuda")
+    gain = torch.ones(Nout, dtype=torch.bfloat16, device="cuda")
+    call = {1: lambda: wide_eng.glance_debug_gemm_wide(1, W, X, terms, act=out),
+            2: lambda: wide_eng.glance_debug_gemm_wide(2, W, X, terms, Y=out, argmax=am),
+            3: lambda: wide_eng.glance_debug_gemm_wide(3, W, X, terms, Y=out, act=act, gain=gain)}[mode]
+    torch.cuda.synchronize()
+    wide_eng.glance_debug_stall_next_gemm(kstep, 100_000)
+    call()
+    assert wide_eng.glance_poll_status() == -5             # GLANCE_E_TIMEOUT
+    assert wide_eng.glance_poll_status() == 0
+    written = torch.zeros(cols, dtype=torch.bool, device="cuda")
+    for lo, hi in done:
+        written[lo:hi] = True
+    assert bool((out[:, ~written] == marker).all()) and (mode != 3 or bool((act == marker).all()))
+    if mode == 1:
+        want = torch.nn.functional.silu(ref[:, :cols]) * ref[:, cols:]
+    else:
+        want = ref + (marker if mode == 3 else 0)
+    bound = (1e-2 if mode == 1 else 1e-4) * float(want.abs().max())
+    assert not done or float((out[:, written].double() - want[:, written]).abs().max()) <= bound
+    call()                                                 # one shot: a normal launch, on the counters the first one left
+    assert wide_eng.glance_poll_status() == 0
+    assert float((out.double() - want).abs().max()) <= bound
+
+
 # ------------------------------------------------------------------ attention alone
 
 def _fill_cache(eng, seq, layer, K, V):
