@@ -245,7 +245,7 @@ int32_t glance_debug_stall_next_gemm(glance_ctx *ctx, int32_t kstep, uint64_t wa
  * n-th GEMM launch after this call makes its first CTA write nanosecond timestamps (entry, set-up done,
  * predecessor finished, first tile landed, accumulator ready, cluster barrier 1, tile shipped, cluster
  * barrier 2, epilogue done, exit) into entries 0-11 of slot n % slots (attention launches count too and record
- * their own phases).  Entries 12-15 are merged over ALL CTAs of the launch with atomic max / min, so the caller
+ * their own phases; the CTA-pair kernel of more than 128 rows records the first item's, without the cluster barriers).  Entries 12-15 are merged over ALL CTAs of the launch with atomic max / min, so the caller
  * presets them (12, 15 to 0; 13, 14 to all ones): 12 = last main loop end, 13 = first main loop end, 14 = first
  * CTA start, 15 = last CTA end.  buffer = NULL, slots = 0 switches it off. */
 int32_t glance_debug_trace(glance_ctx *ctx, uint64_t *buffer, int32_t slots);

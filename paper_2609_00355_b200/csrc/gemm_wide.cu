@@ -322,6 +322,7 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
         const int t = threadIdx.x - 64;
         const uint32_t acc_empty0 = map_to_rank(smem_u32(&bars.acc_empty[0]), 0u);
         bool alive = true;                                // no wait has given up so far (the same in every warp)
+        unsigned long long loop_end = 0;                  // test hook: end of this CTA's main loop so far
         Segment sg;
         for (int i = 0; segment(deal, i, sg); ++i) {
             const int b = i & 1;
@@ -364,6 +365,7 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
             tc_fence_after();
             const uint32_t acc = tmem_base + (uint32_t)b * acc_cols + ((uint32_t)(q * 32) << 16);
             if (trace && t == 0 && i == 0) trace[4] = global_ns();
+            if (a.trace && t == 0) loop_end = global_ns();
             int32_t *counter = a.wide_counters + sg.item * 2 + rank;
             if (n_parts > 1 && t == 0) sh_seen = *reinterpret_cast<volatile int32_t *>(counter);
             // One decision for the CTA; behind this barrier the row scales are there and part_f / part_k are free.  It holds
@@ -644,11 +646,14 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(acc_empty0 + (uint32_t)(b * 8));   // this warp is done with the accumulator
         }
-    }
-    if (trace && threadIdx.x == 64) trace[8] = global_ns();
-    if (a.trace && threadIdx.x == 64) {
-        atomicMin(a.trace + 13, (unsigned long long)global_ns());
-        atomicMax(a.trace + 15, (unsigned long long)global_ns());
+        if (a.trace && t == 0) {
+            if (trace) trace[8] = global_ns();
+            if (loop_end) {                               // (0: this pair had nothing to do)
+                atomicMax(a.trace + 12, loop_end);
+                atomicMin(a.trace + 13, loop_end);
+            }
+            atomicMax(a.trace + 15, (unsigned long long)global_ns());
+        }
     }
     tc_fence_before();
     cluster_sync_all();                                   // neither CTA leaves while the other still uses its memory
@@ -673,6 +678,7 @@ __global__ void __launch_bounds__(NTHR, 1) gemm_wide_kernel(const __grid_constan
         __syncwarp();
         cluster_sync_all();
     }
+    if (trace && threadIdx.x == 0) trace[9] = global_ns();
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(a.tmem_cols) : "memory");

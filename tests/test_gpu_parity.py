@@ -213,6 +213,24 @@ def test_bounded_wait_of_a_pair_runs_out(wide_eng, mode, Nout, K, R, kstep, done
     assert float((out.double() - want).abs().max()) <= bound
 
 
+@pytest.mark.parametrize("Nout,K,R", [(19000, 320, 129), (1000, 2304, 600), (255, 64, 300)])
+def test_trace_of_a_pair_launch(wide_eng, Nout, K, R):
+    """Grid-wide entries as for the 128-row kernel: 12 / 13 the last / first main-loop end, 14 / 15 the launch's span; a
+    launch with entry 12 is what the benchmark counts as a GEMM."""
+    _, W, X, _ = _wide_operands(2, Nout, K, R, 1)
+    am = torch.zeros(R, dtype=torch.int32, device="cuda")
+    buf = torch.zeros(4, 16, dtype=torch.int64, device="cuda")
+    buf[:, 13:15] = torch.iinfo(torch.int64).max
+    torch.cuda.synchronize()
+    wide_eng.glance_debug_trace(buf.view(-1))
+    wide_eng.glance_debug_gemm_wide(2, W, X, argmax=am)
+    assert wide_eng.glance_poll_status() == 0
+    wide_eng.glance_debug_trace(None)
+    t = buf[0].tolist()
+    assert 0 < t[0] <= t[1] <= t[2] <= t[3] <= t[4] <= t[8] <= t[9]
+    assert 0 < t[14] < t[13] <= t[12] <= t[15] and buf[1, 12].item() == 0
+
+
 # ------------------------------------------------------------------ attention alone
 
 def _fill_cache(eng, seq, layer, K, V):
