@@ -64,6 +64,14 @@ constexpr int kPrefillRows = 2048;
 bool use_wide(int mode, int Nout, int K, int R) {
     if (R <= 128 || mode < 1 || mode > 4) return false;
     const WideShape s = wide_shape(mode, Nout, K, R);
+    // Gate/up with one whole round and a rest, where the 128 x 128-row tiles fit one wave of two CTAs per SM: pairs pay for
+    // the rest and its exchange (about 14 us), which long k-loops and a badly filled wave make up for.  Measured at 384 rows
+    // (us a launch, pairs minus tiles): K 2048 with 77 / 89 / 97 % of the wave +3.6 / +9.2 / +10.3, K 3072 97 % +5.8, K 4096
+    // 97 / 81 % +5.9 / -3.9, K 6144 97 % +1.9; at 288 rows 2 to 6 lower.
+    if (mode == 1 && s.rounds == 1 && s.cut > 0) {
+        const int tiles = (Nout / 2 + 63) / 64 * ((R + 127) / 128);
+        if (tiles <= 296 && K / 64 * (1.1 - tiles / 296.0) < 12.0) return false;
+    }
     return s.rounds > 0 ? s.pairs == kWidePairs && K >= 2048 : s.steps >= 48 * kWidePairs;
 }
 
@@ -147,9 +155,12 @@ Workspace carve(const glance_config &c, const Dims &d, unsigned char *base) {
     w.tk_ml = (float *)take(trows * 2 * 4);
     w.tk_cnt = (int32_t *)take(trows * 4);
     w.tk_cand = (unsigned long long *)take(trows * kTopkTileCap * 8);
-    const bool wide = use_wide(4, d.qkv_out, c.hidden, d.Rmax) || use_wide(3, c.hidden, d.qd, d.Rmax) ||
-                      use_wide(1, 2 * c.ffn, c.hidden, d.Rmax) || use_wide(3, c.hidden, c.ffn, d.Rmax) ||
-                      use_wide(2, c.vocab, c.hidden, d.Rlog);
+    bool wide = false;                                  // can any pass choose it?  (the rule sees blocks of 128 rows)
+    for (int r = 256; !wide && r < d.Rmax + 128; r += 128) {
+        const int rows = std::min(r, d.Rmax);
+        wide = use_wide(4, d.qkv_out, c.hidden, rows) || use_wide(3, c.hidden, d.qd, rows) || use_wide(1, 2 * c.ffn, c.hidden, rows) ||
+               use_wide(3, c.hidden, c.ffn, rows) || use_wide(2, c.vocab, c.hidden, std::min(rows, d.Rlog));
+    }
     w.wide_planes = wide ? (float *)take(kWidePlaneFloats * 4) : nullptr;
     w.wide_counters = (int32_t *)take((size_t)kWideCut * 2 * 4);
     w.total = off;

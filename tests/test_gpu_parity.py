@@ -563,10 +563,11 @@ def test_prefill_page_budget_by_groups_of_tree_rows(harness, first, count, statu
     assert written == list(range(first, first + min(count, whole)))
 
 
-@pytest.mark.parametrize("d,ffn,vocab,batch,N", [(64, 2112, 2500, 18, 123), (128, 2112, 2500, 18, 123), (128, 9536, 19000, 3, 43)])
+@pytest.mark.parametrize("d,ffn,vocab,batch,N", [(64, 2112, 2500, 18, 123), (128, 2112, 2500, 18, 123), (128, 9536, 19000, 3, 43),
+                                                   (128, 6144, 2500, 3, 128)])
 def test_batched_pass_equals_single_passes(harness, d, ffn, vocab, batch, N):
     """A verify pass over many rows (CTA-pair GEMMs: whole and cut items, partial last tiles in both directions, one and
-    several row tiles) against the same sequences one by one (128-row GEMMs).  Operands are rounded alike; sums are added
+    several row tiles; gate/up on one full wave of 128-row tiles between them) against the same sequences one by one (128-row GEMMs).  Operands are rounded alike; sums are added
     in another order, which moves a result by at most a bf16 rounding here and there: within the 2e-2 of the other tests."""
     base = synth.CONFIGS["tiny"].replace(n_layers=2, hidden=2112, n_q_heads=2304 // d, n_kv_heads=256 // d, head_dim=d, ffn=ffn,
                                          vocab=vocab, tree_N=N, block_B=4, topk=2)
