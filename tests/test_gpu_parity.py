@@ -492,6 +492,48 @@ def test_walk_commit_examples_and_compaction_hazard(harness):
         assert eng.feat[0, :a + 1, 0].float().tolist() == [float(v) for v in path]
 
 
+@pytest.mark.parametrize("heads,d", [(8, 128), (4, 64)])
+@pytest.mark.parametrize("path", [[0] + list(range(2, 17)), [0] + list(range(1, 16)), [0, 1, 3, 5, 6, 9, 10, 11, 12, 13, 20, 21, 30, 31, 38, 39],
+                                  [0, 4, 5, 6, 7, 8, 9, 39]])
+def test_commit_moves_rows_that_are_both_read_and_written(harness, heads, d, path):
+    """Accepted rows that overlap with their destinations, across a page boundary; eight heads of 128 and 15 steps are 1920
+    16-byte pieces a block, two trips of the copy loop (four of 64: one).  Byte for byte, walk and forced path."""
+    N = 40
+    cfg = synth.CONFIGS["tiny"].replace(n_q_heads=heads, n_kv_heads=heads, head_dim=d, block_B=16, topk=2, tree_N=N)
+    eng = make_engine(cfg, batch=2, max_len=320)
+    a = len(path) - 1
+    for forced in (False, True):
+        lens = [55, 126]
+        g = torch.Generator(device="cuda").manual_seed(a)
+        eng.kv_pool.copy_(torch.randn(eng.kv_pool.shape, generator=g, device="cuda").to(torch.bfloat16))
+        eng.hidden_all.copy_(torch.randn(eng.hidden_all.shape, generator=g, device="cuda").to(torch.bfloat16))
+        eng.seq_len.copy_(torch.tensor(lens, dtype=torch.int32))
+        before = [[torch.stack(eng.gather_kv(s, l, lens[s] + N)).clone() for l in range(cfg.n_layers)] for s in range(2)]
+        if forced:
+            rows = torch.tensor([path + [-1] * (16 - len(path))] * 2, dtype=torch.int32, device="cuda")
+            eng.glance_commit_forced(rows, torch.full((2,), a + 1, dtype=torch.int32, device="cuda"),
+                                     torch.tensor([5, 6], dtype=torch.int32, device="cuda"))
+        else:
+            parent, token = torch.full((N,), -1, dtype=torch.int32), torch.arange(100, 100 + N, dtype=torch.int32)
+            decide = torch.zeros(N, dtype=torch.int32)
+            for u, v in zip(path, path[1:]):
+                parent[v], decide[u] = u, token[v]
+            eng.tree.parent.copy_(parent.expand(2, N)); eng.tree.token.copy_(token.expand(2, N)); eng.tree.n_nodes.fill_(N)
+            eng.argmax.copy_(decide.expand(2, N))
+            eng.glance_accept_commit()
+            assert eng.accept_len.tolist() == [a, a] and eng.path[0, :a + 1].tolist() == path
+        eng.check_device_status()
+        for s in range(2):
+            assert int(eng.seq_len[s]) == lens[s] + a + 1
+            assert torch.equal(eng.feat_all[0, s, :a + 1], eng.hidden_all[0, s, path])
+            for l in range(cfg.n_layers):
+                after = torch.stack(eng.gather_kv(s, l, lens[s] + N))
+                want = before[s][l].clone()
+                for i, v in enumerate(path):
+                    want[:, lens[s] + i] = before[s][l][:, lens[s] + v]
+                assert torch.equal(after, want)
+
+
 def test_commit_forced_and_bad_path_is_reported(harness):
     cfg = synth.CONFIGS["tiny"]
     run = harness.ParityRun(cfg, ctx_lens=[(20, 5)])
@@ -568,7 +610,9 @@ def test_prefill_page_budget_by_groups_of_tree_rows(harness, first, count, statu
 def test_batched_pass_equals_single_passes(harness, d, ffn, vocab, batch, N):
     """A verify pass over many rows (CTA-pair GEMMs: whole and cut items, partial last tiles in both directions, one and
     several row tiles; gate/up on one full wave of 128-row tiles between them) against the same sequences one by one (128-row GEMMs).  Operands are rounded alike; sums are added
-    in another order, which moves a result by at most a bf16 rounding here and there: within the 2e-2 of the other tests."""
+    in another order, so a bf16 result falls on the neighbouring value here and there: at most one unit in the last place
+    (2^-7) of the largest value, and in the 2-norm no more than one rounding of every value (2^-8 / sqrt(3) = 2.3e-3;
+    1.2e-3 was seen).  The entropy follows the logits (7e-5 was seen)."""
     base = synth.CONFIGS["tiny"].replace(n_layers=2, hidden=2112, n_q_heads=2304 // d, n_kv_heads=256 // d, head_dim=d, ffn=ffn,
                                          vocab=vocab, tree_N=N, block_B=4, topk=2)
     from paper_2609_00355_b200.binding import Engine
@@ -612,8 +656,9 @@ def test_batched_pass_equals_single_passes(harness, d, ffn, vocab, batch, N):
     for s in range(batch):
         one = run([s])
         for x, y in ((many[0][s], one[0][0]), (many[1][s], one[1][0]), (many[2][s], one[2][0])):
-            assert float((x - y).abs().max()) <= 2e-2 * float(y.abs().max())
-        assert abs(float(many[3][s] - one[3][0])) <= 1e-3
+            assert float((x - y).abs().max()) <= 2 ** -7 * float(y.abs().max())
+            assert float((x - y).norm()) <= 2.3e-3 * float(y.norm())
+        assert abs(float(many[3][s] - one[3][0])) <= 3e-4
         same += int((many[4][s] == one[4][0]).sum())
     assert same >= 0.95 * batch * N                       # draws differ at near-ties only
 
