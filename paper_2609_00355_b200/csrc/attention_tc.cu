@@ -164,8 +164,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) attn_tc_kernel(const __grid_const
     float sm_w[NG] = {0.f, 0.f};                         // weights of the groups' accumulators in the combined row
 
     if (trace && threadIdx.x == 0) trace[1] = global_ns();
-    // Sequence lengths and page tables only change in the commit kernel of the previous round, long finished:
-    // they may be read before the dependency wait.  Pages entirely below seq_len - block_B hold committed
+    // Sequence lengths change in a commit, a prefill's advance (between its passes too) or a truncation, page tables in the
+    // caller's work, and each of these has finished before any kernel of the pass starts: the pass's row-setup kernel is
+    // launched without programmatic overlap and releases none of its dependents early.  So both may be read before the
+    // dependency wait.  Pages entirely below seq_len - block_B hold committed
     // context that no kernel of this pass writes, so the producer prefetches them before the wait as well.
     const int P = p.seq_len[s];
     // keys any row of this tile sees: all of them, or, in a chain, those up to the tile's last node

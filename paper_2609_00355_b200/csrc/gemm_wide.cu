@@ -13,12 +13,13 @@
 // where the 128 x 128-row tile of gemm_tc_kernel asks for 94 and 128 -- more than the L2 delivers.
 //
 // Persistent: P <= 74 pairs.  Whole rounds of P items (item = weight tile x row tile, row tiles fastest so that concurrent
-// pairs share weight tiles) are dealt out one per pair; the items left over are cut into equal ranges of k-steps, at most
-// eight pairs to an item.  A pair that holds part of an item stores its fp32 partial tile and counts in; the pair that
+// pairs share weight tiles) are dealt out one per pair; the items left over -- all of them, where there are fewer than P --
+// are cut into equal ranges of k-steps, on average at most eight to an item (nine can touch one).  A pair that holds part of an item stores its fp32 partial tile and counts in; the pair that
 // comes last adds the parts in k order (bit-reproducible) and runs the epilogue.  Nobody waits for another pair.  The cut
-// items come first, so that this exchange (20-25 us where nothing follows) hides under the whole ones.  More items than
-// the rest are never cut: pairs at different depths of K share no operands in L2 (the down projection of 1536 rows with
-// all its 84 items cut read 2.4 GB from HBM, 380 us).  Two accumulators in tensor memory: the epilogue of one item runs
+// items come first, so that this exchange (20-25 us where nothing follows) hides under the whole ones.  Where there is a whole
+// round nothing beyond the rest is cut: pairs at different depths of K share no operands in L2 (the down projection of 1536
+// rows with all its 84 items cut read 2.4 GB from HBM, 380 us instead of 288).  A launch of fewer than P items works that way
+// throughout; use_wide() says from how many k-steps a pair on it is still the faster one.  Two accumulators in tensor memory: the epilogue of one item runs
 // under the main loop of the next.
 //
 // Warp roles: warp 0 = TMA producer, warp 1 = tensor memory + MMA issuer (first CTA of the pair), warps 2..9 = epilogue.

@@ -60,7 +60,8 @@ constexpr int kPrefillRows = 2048;
 // outweigh the exchange of partial tiles.  Measured (us, 128 x 128 tiles -> pairs): gate/up 144 / 512 / 1536 rows 102 ->
 // 70, 203 -> 158, 606 -> 480; down 105 -> 53, 178 -> 115 (56 and 112 steps a pair); LM head at 512 rows 582 -> 450; but QKV
 // and O at 512 rows 27 -> 39 and 34 -> 46 (27 and 21 steps), the small model's gate/up at 708 rows 20 -> 31 (14 steps) and, with whole items
-// of only 16 steps each, at 2000 rows 54 -> 57.
+// of only 16 steps each, at 2000 rows 54 -> 57.  At K 2048 an LM head of 32768 gains 9 to 57 us at 130 to 1024 rows; with K 2048
+// to 6144 no pass of 129 to 1024 rows was slower than on the small tiles alone.
 bool use_wide(int mode, int Nout, int K, int R) {
     if (R <= 128 || mode < 1 || mode > 4) return false;
     const WideShape s = wide_shape(mode, Nout, K, R);

@@ -129,6 +129,8 @@ __global__ void __launch_bounds__(128) setup_verify_kernel(VerifySetup p) {
     emit_row(p.out, r, src, p.gain);
 }
 
+// An ordinary launch, and the kernel releases no dependents early: the attention kernels of the pass read sequence lengths
+// and page tables ahead of their own dependency wait and rely on it.  The same holds for launch_setup_draft().
 void launch_setup_verify(const VerifySetup &p, cudaStream_t st) {
     setup_verify_kernel<<<p.batch * p.N, 128, 0, st>>>(p);
 }

@@ -200,12 +200,13 @@ void launch_build_tree(int batch, int N, int L, int k, const int32_t *root, cons
 //
 // Grid (batch, n_layers * 2).  Every block repeats the walk -- all nodes find out in parallel whether their parent's
 // decision names them (the lowest such child of a node is its successor), then one thread follows the successors -- and
-// compacts its own (layer, K|V): cache row P + path[d] -> row P + d for d = 1..a.  Destination row P + d can be the source
-// row of a later step (path is strictly increasing with path[d] >= d), so items go in order of d and a block holds a
-// thousand of them in registers before it stores any.  The block that is the last of its sequence to have read seq_len
+// compacts its own (layer, K|V): cache row P + path[d] -> row P + d for d = 1..a.  Heads are disjoint; within a head items go
+// in ascending d, and path is strictly increasing with path[d] >= d, so a row that a step overwrites can be the source of
+// that step or of an earlier one only.  A block holds a thousand items in registers before it stores any, and a row
+// overwritten in one trip is read by no later one.  The block that is the last of its sequence to have read seq_len
 // publishes the outputs and advances the sequence state; nothing else in the kernel reads what it writes, so nobody waits
-// for the copies.  Eight sequences, 13 rows each, 28 layers: 23.2 -> 6.5 us with a small copy (one block per
-// head made 1.5 waves, each with a walk of warp-wide searches, a fence and a serial publication).
+// for the copies.  Eight sequences, 13 rows each, 28 layers, with a small copy in front: 23.2 -> 6.5 us in a graph, 26.6 ->
+// 18.5 us as two calls of the host (one block per head made 1.5 waves, each with a walk of warp-wide searches, a fence and a serial publication).
 // ------------------------------------------------------------------------------------------
 constexpr int kCommitThreads = 256;
 constexpr int kCommitItems = 4;                          // 16-byte pieces a thread holds at once
