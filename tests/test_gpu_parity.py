@@ -330,6 +330,38 @@ def test_attention_random_inputs(harness, name, P, T):
         assert float((got - ref).abs().max()) <= 2e-2 * float(ref.abs().max())
 
 
+@pytest.mark.parametrize("name,T", [("7b", 1), ("7b", 37), ("small", 16), ("tiny", 65)])
+def test_attention_ends_of_pages_and_tiles(harness, name, T):
+    """Key counts one below, at and one above a whole number of pages, odd and even (a tile of keys is two pages, the last one
+    of a split may have one): one sequence of each in one launch, rows behind the last key poisoned."""
+    cfg = synth.CONFIGS[name].replace(n_layers=1, vocab=256, ffn=64, hidden=64, tree_N=T, n_img=2, n_txt=1, rounds=1)
+    Ps = [max(0, 64 * pages + d - T) for pages in (2, 3, 5, 16) for d in (-1, 0, 1)]
+    eng = make_engine(cfg, batch=len(Ps), max_len=max(Ps) + T + 64)
+    rng, g = np.random.default_rng(T), torch.Generator().manual_seed(T)
+    Hq, Hkv, d = cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim
+    qs, refs, ancs = [], [], []
+    for s, P in enumerate(Ps):
+        tok, par, dep = synth.random_tree(T, 15, 1000, rng)
+        tree = O.tree_from_arrays(tok, par, dep)
+        K = torch.randn(P + T, Hkv, d, generator=g).to(torch.bfloat16)
+        V = torch.randn(P + T, Hkv, d, generator=g).to(torch.bfloat16)
+        q = (torch.randn(T, Hq, d, generator=g) * 1.5).to(torch.bfloat16)
+        eng.seq_len[s] = P
+        poison = torch.full(((-(P + T)) % cfg.page_size, Hkv, d), float("nan"), dtype=torch.bfloat16)
+        _fill_cache(eng, s, 0, torch.cat([K, poison]).cuda(), torch.cat([V, poison]).cuda())
+        refs.append(O.attention(q.float(), K.float(), V.float(), O.visibility(tree, P)))
+        qs.append(q.reshape(T, Hq * d))
+        ancs.append(torch.from_numpy(tree.anc.view(np.int64)))
+    out, out_lo = (torch.zeros(len(Ps) * T, Hq * d, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    eng.glance_debug_attention(0, torch.cat(qs).cuda().contiguous(), torch.stack(ancs).cuda().contiguous(), T, out, out_lo=out_lo)
+    eng.check_device_status()
+    got = (out.float() + out_lo.float()).cpu()
+    for s in range(len(Ps)):
+        # exact bf16 operands, probabilities and outputs of two terms: what is left is fp32 sums and 2^x to 2^-22
+        diff = (got[s * T:(s + 1) * T].reshape(T, Hq, d) - refs[s]).abs().max()
+        assert float(diff) <= 1e-4 * float(refs[s].abs().max()), Ps[s]
+
+
 def test_attention_two_term_queries_and_outputs(harness):
     """fp32 queries given as two bf16 terms, outputs read back as two terms: the only roundings left inside the
     kernel are those of the probabilities and the fp32 accumulation, so the error against the oracle must sit far
