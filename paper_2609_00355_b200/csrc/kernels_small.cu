@@ -385,12 +385,172 @@ __global__ void __launch_bounds__(32) topk_stage2_kernel(int k, int n_warps, con
     }
 }
 
+// ------------------------------------------------------------------------------------------
+// The same in one launch, for rows that the warps of one thread-block cluster hold in registers: a cluster per row, a span
+// of 1024 entries per warp.  What stage 2 reads from scratch meets in the shared memory of the cluster's first CTA, and
+// the log-sum-exp folds the same spans in the same order.  A CTA's bound is the k-th largest of its warps' maxima (k
+// entries reach it), or of a warp's lane maxima where it has fewer than k warps; the few keys that reach it (about 12 of
+// 19000) are ranked by counting the larger ones.  15 rows of 152064, k 8: 18.4 us a call with the two launches (13.8 on the
+// device, the second being 15 single warps over 1192 keys each), 14.7 with this one.  A cluster of eight holds 192 spans in
+// registers; longer rows take the two launches.
+// ------------------------------------------------------------------------------------------
+constexpr int kRowWarps = 24;                            // warps of a CTA at most
+constexpr int kRowCluster = 8;
+constexpr int kRowSpans = kRowWarps * kRowCluster;
+
+// k-th largest of the lanes' values (0 = nothing): one holder leaves per round
+__device__ __forceinline__ uint32_t kth_largest(uint32_t cur, int k, int lane) {
+    uint32_t thr = 0u;
+    for (int t = 0; t < k; ++t) {
+        thr = __reduce_max_sync(0xffffffffu, cur);
+        const uint32_t holders = __ballot_sync(0xffffffffu, cur == thr);
+        if (lane == __ffs(holders) - 1) cur = 0u;
+    }
+    return thr;
+}
+
+__global__ void __launch_bounds__(kRowWarps * 32) topk_row_kernel(const float *logits, int B, int V, int k, int n_spans,
+                                                                  int32_t *ids, float *lp) {
+    constexpr int CAP = 128;                             // keys a CTA collects before it falls back to exact selection
+    __shared__ uint32_t bound[2][kRowWarps];
+    __shared__ unsigned long long list[CAP], best[kMaxTopk], warp_best[kRowWarps];
+    __shared__ int n_list;
+    // in the first CTA: the k best keys of every CTA, and (max, sum of exponentials) of every span
+    __shared__ unsigned long long all[kRowCluster * kMaxTopk];
+    __shared__ __align__(8) float2 span_ml[kRowSpans];
+    const int L = B - 1, row = blockIdx.y, s = row / L, j = row % L + 1;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, warps = blockDim.x >> 5;
+    const int rank = blockIdx.x, ctas = gridDim.x;
+    tc::cluster_arrive();                                // (1) every CTA of the cluster runs: its memory may be written
+    if (tid == 0) n_list = 0;
+    const int span = rank * warps + warp;
+    const float *src = logits + ((size_t)s * B + j) * V;
+    const int base = span * kTopkWarpSpan + lane;
+    float val[32];
+    float m = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        const int c = base + i * 32;
+        val[i] = c < V ? src[c] : -INFINITY;
+        m = fmaxf(m, val[i]);
+    }
+    const float lane_max = m;
+    m = key_float(__reduce_max_sync(0xffffffffu, float_key(lane_max)));
+    // spans behind the row count as empty: 0 is below the image of every value
+    if (lane == 0) bound[0][warp] = span < n_spans ? float_key(m) : 0u;
+    float sum = 0.f;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) sum += expf(val[i] - (m == -INFINITY ? 0.f : m));   // -inf (and entries beyond V) add exactly 0
+    sum = warp_sum(sum);
+    tc::cluster_wait();
+    if (lane == 0 && span < n_spans) {
+        const uint32_t dst = tc::map_to_rank(tc::smem_u32(&span_ml[span]), 0u);
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(m), "f"(sum) : "memory");
+    }
+    __syncthreads();
+    constexpr uint32_t kInf = 0x007fffffu;               // image of -inf
+    uint32_t T = kth_largest(lane < warps ? bound[0][lane] : 0u, k, lane);
+    if (T <= kInf) {                                     // the same in every warp: fewer than k warps, or masked spans
+        const uint32_t mine = kth_largest(span < n_spans ? float_key(lane_max) : 0u, k, lane);
+        if (lane == 0) bound[1][warp] = mine;
+        __syncthreads();
+        T = max(T, __reduce_max_sync(0xffffffffu, lane < warps ? bound[1][lane] : 0u));
+    }
+    if (span < n_spans && float_key(lane_max) >= T) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            const int c = base + i * 32;
+            if (c < V && float_key(val[i]) >= T && val[i] == val[i]) {       // (a NaN is nobody's best)
+                const int at = atomicAdd(&n_list, 1);
+                if (at < CAP) list[at] = pack_val_id(val[i], c);
+            }
+        }
+    }
+    __syncthreads();
+    const int n = n_list;
+    const uint32_t all_here = tc::map_to_rank(tc::smem_u32(&all[rank * k]), 0u);
+    auto give = [&](int r, unsigned long long key) {
+        asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(all_here + 8u * (uint32_t)r), "l"(key) : "memory");
+    };
+    if (n <= CAP) {
+        for (int t = tid; t < max(n, k); t += blockDim.x) {
+            if (t >= n) {                                // fewer than k entries: the other places stay empty
+                give(t, 0ull);
+                continue;
+            }
+            const unsigned long long key = list[t];
+            int r = 0;
+            for (int o = 0; o < n; ++o) r += list[o] > key ? 1 : 0;
+            if (r < k) give(r, key);
+        }
+    } else {
+        // very many equal values at the bound, or fewer than k above -inf: k rounds over everything
+        unsigned long long prev = ~0ull;
+        for (int t = 0; t < k; ++t) {
+            unsigned long long top = 0ull;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const int c = base + i * 32;
+                const unsigned long long key = span < n_spans && c < V ? pack_val_id(val[i], c) : 0ull;
+                if (key < prev && key > top) top = key;
+            }
+            top = warp_max_u64(top);
+            if (lane == 0) warp_best[warp] = top;
+            __syncthreads();
+            for (int w = 0; w < warps; ++w) top = warp_best[w] > top ? warp_best[w] : top;
+            if (tid == 0) give(t, top);
+            prev = top;
+            __syncthreads();
+        }
+    }
+    tc::cluster_sync_all();                              // (2) keys and span statistics are in the first CTA
+    if (rank != 0) return;
+    if (tid < kMaxTopk) best[tid] = 0ull;
+    __syncthreads();
+    for (int t = tid; t < ctas * k; t += blockDim.x) {
+        const unsigned long long key = all[t];
+        int r = 0;
+        for (int o = 0; o < ctas * k; ++o) r += all[o] > key ? 1 : 0;
+        if (key != 0ull && r < k) best[r] = key;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        // log-sum-exp over the spans, fixed order: lane l adds spans l, l + 32, ...; lanes are then summed by shuffles
+        float M = -INFINITY, total = 0.f;
+        for (int w = lane; w < n_spans; w += 32) M = fmaxf(M, span_ml[w].x);
+        M = warp_max(M);
+        for (int w = lane; w < n_spans; w += 32) total += span_ml[w].y * expf(span_ml[w].x - M);
+        total = warp_sum(total);
+        const float lse = M + logf(total);
+        if (lane < k) {
+            ids[(size_t)row * k + lane] = unpack_id(best[lane]);
+            lp[(size_t)row * k + lane] = unpack_val(best[lane]) - lse;
+        }
+    }
+}
+
 int topk_warps(int V) { return (V + kTopkWarpSpan - 1) / kTopkWarpSpan; }
 
 void launch_topk(const float *logits, int batch, int B, int V, int k, int32_t *ids, float *lp,
                  unsigned long long *cand, float *ml, cudaStream_t st) {
     if (B < 2) return;
     const int rows = batch * (B - 1), nw = topk_warps(V);
+    if (nw <= kRowSpans) {
+        const int ctas = nw > 8 ? kRowCluster : 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(ctas, rows, 1);
+        cfg.blockDim = dim3(32 * ((nw + ctas - 1) / ctas), 1, 1);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = ctas;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cudaLaunchKernelEx(&cfg, topk_row_kernel, logits, B, V, k, nw, ids, lp);
+        return;
+    }
     dim3 g1((nw + 3) / 4, rows);
     topk_stage1_kernel<<<g1, 128, 0, st>>>(logits, B, V, k, nw, cand, ml);
     topk_stage2_kernel<<<rows, 32, 0, st>>>(k, nw, cand, ml, ids, lp);

@@ -77,7 +77,9 @@ def test_topk_static_matches_draft_block_and_oracle_twice():
 
 @pytest.mark.parametrize("V,k,kind", [(2, 1, "random"), (16, 16, "random"), (1000, 7, "ties"), (1025, 16, "random"), (33000, 16, "ties"),
                                       (262144, 16, "random"), (262145, 3, "random"), (600000, 16, "random"), (600000, 16, "stripes"),
-                                      (70000, 5, "inf")])
+                                      (70000, 5, "inf"),
+                                      # one CTA and a cluster of them, and the last vocabulary that a cluster takes
+                                      (8192, 16, "random"), (8193, 16, "ties"), (9000, 16, "inf"), (196608, 16, "random"), (196609, 2, "ties")])
 def test_topk_static_edges_of_spans_and_lists(V, k, kind):
     """One span, its remainders, more spans than threads, many equal values, -inf entries, and keys concentrated in a few
     spans, against the exact (logit desc, id asc) order on the CPU."""
