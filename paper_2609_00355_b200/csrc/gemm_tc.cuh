@@ -71,7 +71,7 @@ struct TcGemmArgs {
     // [kWideCut][2] (zero between launches)
     float *wide_planes;
     int32_t *wide_counters;
-    int wide_pairs, wide_row_tiles, wide_rounds, wide_cut, wide_cutters;      // filled by launch_gemm_wide
+    int wide_pairs, wide_row_tiles, wide_rounds, wide_cut, wide_cutters, wide_items;      // filled by launch_gemm_wide
     // filled by launch_gemm_tc / launch_gemm_wide
     int np, stages, rows_fastest;
     uint32_t tmem_cols;

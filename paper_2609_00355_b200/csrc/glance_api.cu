@@ -69,11 +69,11 @@ bool use_wide(int mode, int Nout, int K, int R) {
     // the rest and its exchange (about 14 us), which long k-loops and a badly filled wave make up for.  Measured at 384 rows
     // (us a launch, pairs minus tiles): K 2048 with 77 / 89 / 97 % of the wave +3.6 / +9.2 / +10.3, K 3072 97 % +5.8, K 4096
     // 97 / 81 % +5.9 / -3.9, K 6144 97 % +1.9; at 288 rows 2 to 6 lower.
-    if (mode == 1 && s.rounds == 1 && s.cut > 0) {
+    if (mode == 1 && s.items / s.pairs == 1 && s.items % s.pairs > 0) {
         const int tiles = (Nout / 2 + 63) / 64 * ((R + 127) / 128);
         if (tiles <= 296 && K / 64 * (1.1 - tiles / 296.0) < 12.0) return false;
     }
-    return s.rounds > 0 ? s.pairs == kWidePairs && K >= 2048 : s.steps >= 48 * kWidePairs;
+    return s.items >= s.pairs ? s.pairs == kWidePairs && K >= 2048 : s.steps >= 48 * kWidePairs;
 }
 
 struct Workspace {

@@ -139,7 +139,9 @@ def _wide_operands(mode, Nout, K, R, terms):
 @pytest.mark.parametrize("mode,Nout,K,R,terms", [
     (1, 1408, 2304, 200, 2), (1, 20480, 256, 130, 2), (1, 128, 64, 129, 1), (1, 4096, 1024, 1000, 2),
     (2, 19000, 320, 129, 1), (2, 1000, 2304, 600, 1), (2, 255, 64, 300, 1), (2, 18945, 1024, 256, 1),
-    (3, 2304, 8192, 144, 2), (3, 2112, 4096, 1024, 2), (3, 64, 64, 129, 1), (3, 192, 2304, 300, 2)])
+    (3, 2304, 8192, 144, 2), (3, 2112, 4096, 1024, 2), (3, 64, 64, 129, 1), (3, 192, 2304, 300, 2),
+    # 66 items: a rest that nearly fills a round is dealt out whole
+    (1, 8448, 1024, 300, 2)])
 def test_gemm_wide(wide_eng, mode, Nout, K, R, terms):
     """CTA-pair GEMM against a 64-bit matmul of the same bf16 terms: the bounds of the 128-row kernel's tests, sums in fp32
     (1e-4 of the largest result), act one bf16 rounding of it (eight significant bits: half a unit in the last place is at
