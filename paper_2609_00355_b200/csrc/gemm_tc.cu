@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
     const int tile_idx = a.rows_fastest ? blockIdx.z : blockIdx.x;
     const int f0 = tile_idx * FT;
     const int split = blockIdx.y;
-    const int r0 = (a.rows_fastest ? blockIdx.x : blockIdx.z) * 128;
+    const int r0 = (a.rows_fastest ? blockIdx.x : blockIdx.z) * NP;
     const int xr0 = r0 + a.x_row0;                       // first row inside X
     const int ktiles = a.K / BK;
     const int kt0 = (int)((long long)split * ktiles / a.S), kt1 = (int)((long long)(split + 1) * ktiles / a.S);
@@ -218,40 +218,49 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     const uint32_t rank = CLUSTERED ? cluster_rank() : 0u;
     const int RP = CLUSTERED ? (NP + a.S - 1) / a.S : NP; // rows per owner CTA
-    // Rows this CTA finishes (all NP, or its band of the cluster's reduce-scatter) and, for the first two rows
-    // of each epilogue warp, the global operands of the row processing (residual, gain, rotary table, K/V row):
-    // they are fetched here, ahead of the merge, so that their L2 latency hides under it.
+    // Rows this CTA finishes (all NP, or its band of the cluster's reduce-scatter).  The global operands of the row
+    // processing (residual, rotary table, K/V row) are fetched ahead: those of a warp's first rows before the merge, under
+    // which they travel.  Mode 3 then takes four rows at a time, one L2 latency for all of them (O at 577 rows, 8 rows a warp:
+    // 19.7 -> 15.4 us); mode 4, whose body written out four times is slower than what it saves (every launch finds its
+    // instructions cold: QKV at 512 rows 28.9 -> 31.5 us), stays rolled and fetches a row's operands one row ahead.
     const int ew = warp - 2;                             // epilogue warp 0..7
     const int row_lo = (int)rank * RP;                   // first owned row (tile-local)
     const int my_rows = max(0, min(min(RP, NP - row_lo), a.R - r0 - row_lo));
     const int fo = 4 * lane;                             // first of this thread's four features (tile-local)
-    float4 pre_a[2], pre_b[2], gain = make_float4(0.f, 0.f, 0.f, 0.f);
-    long long pre_kv[2] = {-1, -1};
-    pre_a[0] = pre_a[1] = pre_b[0] = pre_b[1] = gain;
-    if (warp >= 2 && f0 + fo < a.Nout) {
+    constexpr int BATCH = MODE == 3 ? 4 : 2, EARLY = 2;
+    float4 pre_a[BATCH], pre_b[BATCH], gain = make_float4(0.f, 0.f, 0.f, 0.f);
+    long long pre_kv[BATCH];
+    auto fetch = [&](int u, int lr) {
+        if (lr >= my_rows || f0 + fo >= a.Nout) return;
+        const int rr = r0 + row_lo + lr;
         if (MODE == 3) {
-            const uint2 gg = *reinterpret_cast<const uint2 *>(a.gain + f0 + fo);
-            const __nv_bfloat162 g01 = *reinterpret_cast<const __nv_bfloat162 *>(&gg.x);
-            const __nv_bfloat162 g23 = *reinterpret_cast<const __nv_bfloat162 *>(&gg.y);
-            gain = make_float4(__low2float(g01), __high2float(g01), __low2float(g23), __high2float(g23));
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-                if (ew + u * NEPI < my_rows)
-                    pre_a[u] = __ldcg(reinterpret_cast<const float4 *>(a.x + (size_t)(r0 + row_lo + ew + u * NEPI) * a.Nout + f0 + fo));
-        } else if (MODE == 4) {
+            pre_a[u] = __ldcg(reinterpret_cast<const float4 *>(a.x + (size_t)rr * a.Nout + f0 + fo));
+        } else {
             const int d = a.head_dim, half = d >> 1;
             const int h = (f0 + fo) / d, i = (f0 + fo) % d;
             const int ci = (i < half) ? i : i - half;
+            if (h < a.Hq + a.Hkv) {
+                pre_a[u] = *reinterpret_cast<const float4 *>(a.rope_cos + (size_t)rr * half + ci);
+                pre_b[u] = *reinterpret_cast<const float4 *>(a.rope_sin + (size_t)rr * half + ci);
+            }
+            if (h >= a.Hq) pre_kv[u] = a.kvrow[rr];
+        }
+    };
+    if (CLUSTERED) {
 #pragma unroll
-            for (int u = 0; u < 2; ++u)
-                if (ew + u * NEPI < my_rows) {
-                    const int rr = r0 + row_lo + ew + u * NEPI;
-                    if (h < a.Hq + a.Hkv) {
-                        pre_a[u] = *reinterpret_cast<const float4 *>(a.rope_cos + (size_t)rr * half + ci);
-                        pre_b[u] = *reinterpret_cast<const float4 *>(a.rope_sin + (size_t)rr * half + ci);
-                    }
-                    if (h >= a.Hq) pre_kv[u] = a.kvrow[rr];
-                }
+        for (int u = 0; u < BATCH; ++u) {
+            pre_a[u] = pre_b[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            pre_kv[u] = -1;
+        }
+        if (warp >= 2) {
+            if (MODE == 3 && f0 + fo < a.Nout) {
+                const uint2 gg = *reinterpret_cast<const uint2 *>(a.gain + f0 + fo);
+                const __nv_bfloat162 g01 = *reinterpret_cast<const __nv_bfloat162 *>(&gg.x);
+                const __nv_bfloat162 g23 = *reinterpret_cast<const __nv_bfloat162 *>(&gg.y);
+                gain = make_float4(__low2float(g01), __high2float(g01), __low2float(g23), __high2float(g23));
+            }
+#pragma unroll
+            for (int u = 0; u < EARLY; ++u) fetch(u, ew + u * NEPI);
         }
     }
     if (CLUSTERED) {
@@ -487,36 +496,33 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
         } else if (MODE == 3) {
             const int f = f0 + fo;
             const bool valid = f < a.Nout;               // Nout is a multiple of 4
-            int it = 0;
-            for (int lr = ew; lr < my_rows; lr += NEPI, ++it) {
-                const size_t o = (size_t)(r0 + row_lo + lr) * a.Nout + f;
-                float4 xv = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (it == 0) xv = pre_a[0];
-                else if (it == 1) xv = pre_a[1];
-                else if (valid) xv = __ldcg(reinterpret_cast<const float4 *>(a.x + o));
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int k = 0; k < a.S; ++k) {          // split order: bit-reproducible
-                    const float4 p = *reinterpret_cast<const float4 *>(tile + (size_t)(k * RP + lr) * BM + fo);
-                    v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
-                }
-                float sq = 0.f;
-                if (valid) {
-                    xv.x += v.x; xv.y += v.y; xv.z += v.z; xv.w += v.w;
-                    *reinterpret_cast<float4 *>(a.x + o) = xv;
-                    store_two_term(a.xb + o, a.xb_lo ? a.xb_lo + o : nullptr,
-                                   make_float4(xv.x * gain.x, xv.y * gain.y, xv.z * gain.z, xv.w * gain.w));
-                    if (a.hidden_out) {
-                        uint2 ob;
-                        __nv_bfloat162 lo = __floats2bfloat162_rn(xv.x, xv.y);
-                        __nv_bfloat162 hi = __floats2bfloat162_rn(xv.z, xv.w);
-                        ob.x = *reinterpret_cast<uint32_t *>(&lo);
-                        ob.y = *reinterpret_cast<uint32_t *>(&hi);
-                        *reinterpret_cast<uint2 *>(a.hidden_out + o) = ob;
+            for (int lr0 = ew; lr0 < my_rows; lr0 += BATCH * NEPI) {
+#pragma unroll
+                for (int u = 0; u < BATCH; ++u)
+                    if (lr0 != ew || u >= EARLY) fetch(u, lr0 + u * NEPI);
+#pragma unroll
+                for (int u = 0; u < BATCH; ++u) {
+                    const int lr = lr0 + u * NEPI;
+                    if (lr >= my_rows) break;
+                    const size_t o = (size_t)(r0 + row_lo + lr) * a.Nout + f;
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int k = 0; k < a.S; ++k) {      // split order: bit-reproducible
+                        const float4 p = *reinterpret_cast<const float4 *>(tile + (size_t)(k * RP + lr) * BM + fo);
+                        v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
                     }
-                    sq = ((xv.x * xv.x + xv.y * xv.y) + xv.z * xv.z) + xv.w * xv.w;
+                    float sq = 0.f;
+                    if (valid) {
+                        float4 xv = pre_a[u];
+                        xv.x += v.x; xv.y += v.y; xv.z += v.z; xv.w += v.w;
+                        *reinterpret_cast<float4 *>(a.x + o) = xv;
+                        store_two_term(a.xb + o, a.xb_lo ? a.xb_lo + o : nullptr,
+                                       make_float4(xv.x * gain.x, xv.y * gain.y, xv.z * gain.z, xv.w * gain.w));
+                        if (a.hidden_out) store_two_term(a.hidden_out + o, nullptr, xv);
+                        sq = ((xv.x * xv.x + xv.y * xv.y) + xv.z * xv.z) + xv.w * xv.w;
+                    }
+                    sq = warp_sum(sq);                   // one warp spans the tile's 128 features
+                    if (lane == 0) a.ssq_out[(size_t)tile_idx * a.ssq_stride + r0 + row_lo + lr] = sq;
                 }
-                sq = warp_sum(sq);                       // one warp spans the tile's 128 features
-                if (lane == 0) a.ssq_out[(size_t)tile_idx * a.ssq_stride + r0 + row_lo + lr] = sq;
             }
         } else {
             // MODE 4: q heads, then k heads, then v heads; rotary pairs (i, i + d/2) lie in the same tile
@@ -528,9 +534,13 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
             const int pfo = (i < half) ? fo + half : fo - half;
             const int ci = (i < half) ? i : i - half;
             const int kvh = is_k ? h - a.Hq : h - a.Hq - a.Hkv;
-            int it = 0;
-            for (int lr = ew; lr < my_rows; lr += NEPI, ++it) {
+#pragma unroll 1
+            for (int lr = ew; lr < my_rows; lr += NEPI) {
                 const int rr = r0 + row_lo + lr;
+                const float4 cs = pre_a[0], sn = pre_b[0];
+                const long long base = pre_kv[0];
+                pre_a[0] = pre_a[1]; pre_b[0] = pre_b[1]; pre_kv[0] = pre_kv[1];
+                fetch(1, lr + 2 * NEPI);                 // two rows ahead: nothing below waits for it
                 float4 va = make_float4(0.f, 0.f, 0.f, 0.f), vb = va;
                 for (int k = 0; k < a.S; ++k) {
                     const float *pl = tile + (size_t)(k * RP + lr) * BM;
@@ -545,8 +555,6 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
                 vb.x *= sc; vb.y *= sc; vb.z *= sc; vb.w *= sc;
                 float4 out = va;
                 if (is_q || is_k) {
-                    const float4 cs = it == 0 ? pre_a[0] : it == 1 ? pre_a[1] : *reinterpret_cast<const float4 *>(a.rope_cos + (size_t)rr * half + ci);
-                    const float4 sn = it == 0 ? pre_b[0] : it == 1 ? pre_b[1] : *reinterpret_cast<const float4 *>(a.rope_sin + (size_t)rr * half + ci);
                     if (i < half) {
                         out.x = va.x * cs.x - vb.x * sn.x; out.y = va.y * cs.y - vb.y * sn.y;
                         out.z = va.z * cs.z - vb.z * sn.z; out.w = va.w * cs.w - vb.w * sn.w;
@@ -559,14 +567,8 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
                     // queries keep two bf16 terms: their rounding error would otherwise reach every score of the row
                     const size_t qo = ((size_t)rr * a.Hq + h) * d + i;
                     if (rr < a.Rq) store_two_term(a.q + qo, a.q_lo ? a.q_lo + qo : nullptr, out);
-                } else {
-                    __nv_bfloat162 lo = __floats2bfloat162_rn(out.x, out.y), hi = __floats2bfloat162_rn(out.z, out.w);
-                    uint2 ob;
-                    ob.x = *reinterpret_cast<uint32_t *>(&lo);
-                    ob.y = *reinterpret_cast<uint32_t *>(&hi);
-                    const long long base = it == 0 ? pre_kv[0] : it == 1 ? pre_kv[1] : a.kvrow[rr];
-                    if (base >= 0)
-                        *reinterpret_cast<uint2 *>(a.pool_layer + (size_t)base + (is_k ? 0 : a.v_off) + (size_t)kvh * a.head_stride + i) = ob;
+                } else if (base >= 0) {
+                    store_two_term(a.pool_layer + (size_t)base + (is_k ? 0 : a.v_off) + (size_t)kvh * a.head_stride + i, nullptr, out);
                 }
             }
         }
@@ -655,9 +657,10 @@ bool tc_make_map_nd(CUtensorMap *map, const void *base, int n, const uint64_t *d
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Equal row blocks: 144 rows are two blocks of 80 (padded), not 128 and 16.
 int tc_row_pad(int R) {
-    const int r = R > 128 ? 128 : R;
-    return (r + 15) / 16 * 16;
+    const int blocks = (R + 127) / 128;
+    return ((R + blocks - 1) / blocks + 15) / 16 * 16;
 }
 
 cudaError_t launch_gemm_tc(int mode, TcGemmArgs a, const CUtensorMap &map_w, const CUtensorMap &map_x, cudaStream_t st) {
@@ -671,14 +674,18 @@ cudaError_t launch_gemm_tc(int mode, TcGemmArgs a, const CUtensorMap &map_w, con
     // The LM heads have a few more tiles than two CTAs per SM take in four rounds (1188 against 1184 at the 7B
     // vocabulary): with a smaller ring three CTAs fit per SM and the last round is as full as the others.
     const bool three = (mode == 0 || mode == 2 || mode == 5) && tiles > 3 * 148;
-    int stages = (int)(((three ? 72 : 100) * 1024) / stage_bytes);
+    // A launch of at most one CTA per SM takes a whole SM's ring: more of its weights, often all of them, are fetched before
+    // the dependency wait (gate/up of 131 rows, h 1024, 88 CTAs: 13.6 -> 9.5 us).  With more CTAs the same ring would cost the
+    // second CTA of an SM (down of the 7B widths, S 5: 23.5 -> 44 us).
+    const int row_blocks = (a.R + 127) / 128;
+    const bool alone = mode != 0 && !three && tiles * a.S * row_blocks <= 148;
+    int stages = (int)(((three ? 72 : alone ? 200 : 100) * 1024) / stage_bytes);
     stages = stages > 12 ? 12 : (stages < 2 ? 2 : stages);
     a.stages = stages;
     uint32_t cols = 32;
     while ((int)cols < nb) cols <<= 1;
     a.tmem_cols = cols;
     const size_t smem = (size_t)stages * stage_bytes + 1024;
-    const int row_blocks = (a.R + 127) / 128;
     a.rows_fastest = row_blocks > 1 ? 1 : 0;
     dim3 grid(a.rows_fastest ? row_blocks : tiles, a.S, a.rows_fastest ? tiles : row_blocks);
     if (mode == 3 || mode == 4) {

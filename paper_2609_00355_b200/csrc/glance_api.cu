@@ -27,24 +27,27 @@ int choose_split(int Nout, int K, int rows, bool two_term) {
     const int ktiles = K / 64;
     const int row_blocks = (rows + 127) / 128;
     if (row_blocks > 1) {
-        // Two CTAs per SM keep about 200 KB of operands in flight, which is what the tensor rate needs from L2; one
-        // CTA per SM runs at about half of it.  So a wave is 296 items wide, each item running at half an SM's rate.
-        const double step_us = two_term ? 0.45 : 0.225;       // one 128 x 128-row x 64 k-step at an SM's tensor rate
-        const double unit_us = ktiles * step_us;               // one unsplit item with the SM to itself
-        const int smax = std::max(1, std::min(8, ktiles / 7));
+        // A k-step of a CTA is bound by the arrival of its operands, and the exchange at the end costs about the same
+        // whatever the split (us, one 7B layer: QKV at 144 rows S = 1 / 2 / 3 / 4: 35 / 22 / 18 / 29, O 45 / 27 / 21 / 18 and 26
+        // with five; 256 rows: QKV 43 / 27 / 23 / 35, O 54 / 32 / 25 / 22 and 30).  The jumps are launches that no longer fit
+        // at once: 296 CTAs are resident without clusters or in pairs, about 250 in larger clusters -- which a long loop makes up
+        // for (down, 56 tiles and blocks, four and five splits: 59 / 53 at 144 rows, 79 / 61 at 256).
+        const double step_us = 0.29 + 0.002 * tc_row_pad(rows) * (two_term ? 2 : 1);
+        const int smax = std::max(1, std::min(8, ktiles / 2));
         int best = 1;
         double best_us = 1e30;
         for (int s = 1; s <= smax; ++s) {
-            const double waves = std::ceil((double)tiles * row_blocks * s / 296.0);
-            // cluster epilogue per wave; clusters of a later wave also wait for enough SMs of one GPC to come free together
-            const double epilogue_us = s == 1 ? 0.0 : (waves > 1.0 ? 10.0 : 3.0);
-            const double us = waves * (2.0 * unit_us / s + epilogue_us);
+            const double waves = std::ceil((double)tiles * row_blocks * s / (s <= 2 || ktiles >= 40 * s ? 296.0 : 250.0));
+            const double us = waves * (ktiles * step_us / s + 9.5);
             if (us < best_us - 1e-9) { best_us = us; best = s; }
         }
         return best;
     }
     int s = (2 * 148) / tiles;
     s = std::min(s, std::max(1, ktiles / 7));
+    // a launch of few CTAs: more and shorter splits, whose weights are all fetched before the predecessor is done (small model,
+    // h 1024, 32 rows, QKV / O / down: 7.5 / 7.5 / 7.4 us with 2 / 2 / 6 splits, 6.4 / 5.3 / 6.8 with eight and whole rings)
+    s = std::max(s, std::min(148 / tiles, ktiles / 2));
     s = std::max(1, std::min(s, 8));
     if (s == 8 && tiles > 33) s = 7;                   // at most 33 clusters of eight are resident at two CTAs per SM
     return s;
@@ -58,9 +61,10 @@ constexpr int kPrefillRows = 2048;
 // Whether a GEMM over more than 128 rows runs on CTA pairs with 256 x 256 tiles (gemm_wide.cu) or on the 128 x 128-row
 // tiles of gemm_tc_kernel.  It does where every pair has at least one whole item, or where the k-steps of a pair's share
 // outweigh the exchange of partial tiles.  Measured (us, 128 x 128 tiles -> pairs): gate/up 144 / 512 / 1536 rows 102 ->
-// 70, 203 -> 158, 606 -> 480; down 105 -> 53, 178 -> 115 (56 and 112 steps a pair); LM head at 512 rows 582 -> 450; but QKV
+// 70, 203 -> 158, 606 -> 480; down at 512 rows 178 -> 111 (112 steps a pair); LM head at 512 rows 582 -> 450; but QKV
 // and O at 512 rows 27 -> 39 and 34 -> 46 (27 and 21 steps), the small model's gate/up at 708 rows 20 -> 31 (14 steps) and, with whole items
-// of only 16 steps each, at 2000 rows 54 -> 57.  At K 2048 an LM head of 32768 gains 9 to 57 us at 130 to 1024 rows; with K 2048
+// of only 16 steps each, at 2000 rows 54 -> 57.  Where an item would have more than four parts the exchange eats the gain
+// (down at 256 rows, 14 items: 61 on tiles, 74 on pairs; at 144 rows 51 and 53).  At K 2048 an LM head of 32768 gains 9 to 57 us at 130 to 1024 rows; with K 2048
 // to 6144 no pass of 129 to 1024 rows was slower than on the small tiles alone.
 bool use_wide(int mode, int Nout, int K, int R) {
     if (R <= 128 || mode < 1 || mode > 4) return false;
@@ -73,7 +77,7 @@ bool use_wide(int mode, int Nout, int K, int R) {
         const int tiles = (Nout / 2 + 63) / 64 * ((R + 127) / 128);
         if (tiles <= 296 && K / 64 * (1.1 - tiles / 296.0) < 12.0) return false;
     }
-    return s.items >= s.pairs ? s.pairs == kWidePairs && K >= 2048 : s.steps >= 48 * kWidePairs;
+    return s.items >= s.pairs ? s.pairs == kWidePairs && K >= 2048 : 4 * s.items >= s.pairs && s.steps >= 48 * kWidePairs;
 }
 
 struct Workspace {

@@ -60,6 +60,24 @@ def test_gemm_tc_planes(gemm_eng, Nout, K, R, S):
     assert torch.equal(Y, Y2)
 
 
+@pytest.mark.parametrize("R", [129, 144, 257, 270])
+def test_gemm_tc_equal_row_blocks(gemm_eng, R):
+    """More than one row block: blocks of equal height (padded to 16), the last one with rows to spare."""
+    if R > 256:
+        eng = make_engine(synth.CONFIGS["tiny"].replace(tree_N=128, vocab=256), batch=3)
+    else:
+        eng = gemm_eng
+    g = torch.Generator(device="cuda").manual_seed(R)
+    Nout, K, S = 300, 320, 2
+    W = (torch.randn(Nout, K, generator=g, device="cuda") * 0.05).to(torch.bfloat16)
+    X = torch.randn(R, K, generator=g, device="cuda").to(torch.bfloat16)
+    Y = torch.full((S, R, Nout), float("nan"), device="cuda")
+    eng.glance_debug_gemm(0, W, X, Y=Y, S=S)
+    assert eng.glance_poll_status() == 0
+    ref = X.double() @ W.double().T
+    assert float((Y.double().sum(0) - ref).abs().max()) <= 1e-4 * float(ref.abs().max()) + 1e-5
+
+
 def test_bounded_wait_runs_out_and_the_context_stays_usable(gemm_eng):
     """Failure detection on the device, without a fault: one ring slot of a tiny GEMM is never filled (chosen on the
     host), the MMA issuer's bounded wait on it gives up after 100 us, the CTA drains the copies it has in flight,
@@ -140,8 +158,9 @@ def _wide_operands(mode, Nout, K, R, terms):
     (1, 1408, 2304, 200, 2), (1, 20480, 256, 130, 2), (1, 128, 64, 129, 1), (1, 4096, 1024, 1000, 2),
     (2, 19000, 320, 129, 1), (2, 1000, 2304, 600, 1), (2, 255, 64, 300, 1), (2, 18945, 1024, 256, 1),
     (3, 2304, 8192, 144, 2), (3, 2112, 4096, 1024, 2), (3, 64, 64, 129, 1), (3, 192, 2304, 300, 2),
-    # 66 items: a rest that nearly fills a round is dealt out whole
-    (1, 8448, 1024, 300, 2)])
+    # shared items handed over by groups of rows: more and fewer parts than steps of 32 rows, rows that end inside a group;
+    # 66 items, a rest that is dealt out whole
+    (3, 512, 8192, 129, 2), (3, 1024, 8192, 250, 2), (2, 512, 8192, 161, 1), (1, 8448, 1024, 300, 2)])
 def test_gemm_wide(wide_eng, mode, Nout, K, R, terms):
     """CTA-pair GEMM against a 64-bit matmul of the same bf16 terms: the bounds of the 128-row kernel's tests, sums in fp32
     (1e-4 of the largest result), act one bf16 rounding of it (eight significant bits: half a unit in the last place is at
