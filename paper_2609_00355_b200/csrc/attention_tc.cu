@@ -730,8 +730,8 @@ int attention_tc_q_tiles(int T, int G) { return (T * G + QT - 1) / QT; }
 // launch should be resident at once (a second wave would double the kernel's latency).  A launch that cannot fit
 // one wave split (several sequences) gets two splits: that halves the longest sequence's loop, which sets the
 // launch's duration, while larger clusters lose more than they gain once clusters queue for SMs (a cluster starts
-// only when enough SMs of one GPC are free together: 8 sequences of 1024-4096 positions took 100 / 84 / 102 / 154 us
-// per layer with 1 / 2 / 4 / 8 splits).
+// only when enough SMs of one GPC are free together: with 64-key tiles 8 sequences of 1024-4096 positions took 100 / 84 /
+// 102 / 154 us per layer with 1 / 2 / 4 / 8 splits; with 128-key tiles two splits take 70).
 int attention_tc_splits(int T, int G, int Hkv, int batch, int d) {
     const int base = attention_tc_q_tiles(T, G) * Hkv * batch;
     for (int s = MAX_SPLITS; s > 1; --s) {

@@ -10,7 +10,7 @@ namespace glance {
 
 typedef __nv_bfloat16 bf16;
 
-constexpr int kPage = 64;        // tokens per KV page (one 64-key attention tile = one page)
+constexpr int kPage = 64;        // tokens per KV page (an attention tile is two pages)
 constexpr int kMaxTreeN = 128;   // verify rows per sequence, root included
 constexpr int kMaxTopk = 16;
 constexpr int kMaxBlock = 16;

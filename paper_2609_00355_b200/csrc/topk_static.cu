@@ -5,8 +5,9 @@
 // a plug-in running inside a host framework's callback where allocation calls are off limits, or a
 // latency-critical loop that cannot tolerate the implicit device-wide synchronisation an allocation may
 // cause.  The regular path asks such callers for a workspace sized by glance_workspace_bytes(); this
-// entry point needs none: the two-stage top-k keeps its per-warp candidates and partial log-sum-exp
-// terms in the file-scope array below, which every GPU that loads the library holds until the process exits.
+// entry point needs none.  Rows of up to 192 spans of 1024 entries are merged in the shared memory of a thread-block cluster;
+// for longer ones the two-stage top-k keeps its per-warp candidates and partial log-sum-exp terms in the file-scope array
+// below, which every GPU that loads the library holds until the process exits.  Its size bounds every request.
 #include <mutex>
 
 #include "kernels.cuh"
