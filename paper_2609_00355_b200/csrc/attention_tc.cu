@@ -87,10 +87,12 @@ struct Smem {
     // behind them the rows received (each owner gets <= ceil(QT/S) rows from each of S CTAs)
     static constexpr int RECV_AT = QT * ROWF * 4;
     static constexpr int RECV_BYTES = (QT + MAX_SPLITS) * ROWF * 4;
-    static constexpr int TOTAL = OPER_BYTES + 1024;
     // tensor memory columns: one S/P buffer of 128 and one accumulator (d) per group
     static constexpr uint32_t O_COL = NG * KT;
     static constexpr uint32_t TMEM_COLS = 512;
+    // d 64 would fit twice into an SM's shared memory, and clusters whose CTAs hold the columns crosswise would wait for each
+    // other in a cluster barrier
+    static constexpr int TOTAL = OPER_BYTES + 1024 > (int)least_smem(TMEM_COLS) ? OPER_BYTES + 1024 : (int)least_smem(TMEM_COLS);
     static_assert(O_COL + NG * D <= TMEM_COLS, "tensor memory budget");
     static_assert(RECV_AT + RECV_BYTES <= OPER_BYTES, "the merge fits the operand buffers");
     static_assert(RECV_AT % 16 == 0 && ROWF % 4 == 0, "bulk copies start on 16-byte boundaries");
@@ -723,6 +725,10 @@ int max_active_clusters(int cs) {
 }
 
 }  // namespace
+
+CtaSize attention_tc_cta_size(int d) {
+    return d == 128 ? CtaSize{Smem<128>::TOTAL, Smem<128>::TMEM_COLS} : CtaSize{Smem<64>::TOTAL, Smem<64>::TMEM_COLS};
+}
 
 int attention_tc_q_tiles(int T, int G) { return (T * G + QT - 1) / QT; }
 

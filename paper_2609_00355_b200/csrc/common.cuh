@@ -10,6 +10,11 @@ namespace glance {
 
 typedef __nv_bfloat16 bf16;
 
+// what one CTA of a launch asks for: bytes of dynamic shared memory, columns of tensor memory
+struct CtaSize {
+    long long smem, columns;
+};
+
 constexpr int kPage = 64;        // tokens per KV page (an attention tile is two pages)
 constexpr int kMaxTreeN = 128;   // verify rows per sequence, root included
 constexpr int kMaxTopk = 16;

@@ -127,6 +127,7 @@ struct AttnParams {
 };
 // map_kv = 2-D map of the pool layer {d, n_pages*2*Hkv*64 rows}, box {64, 64}
 cudaError_t launch_attention_tc(const AttnParams &p, const CUtensorMap &map_kv, cudaStream_t st);
+CtaSize attention_tc_cta_size(int d);
 int attention_tc_q_tiles(int T, int G);
 int attention_tc_splits(int T, int G, int Hkv, int batch, int d);
 

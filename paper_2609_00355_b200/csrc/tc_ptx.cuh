@@ -11,6 +11,14 @@ namespace tc {
 constexpr int BM = 128;
 constexpr int BK = 64;
 
+// Who may share an SM.  tcgen05.alloc blocks until its columns are free, and their holder may itself be waiting: for an earlier
+// kernel (programmatic dependent launch) or for a CTA of its cluster, neither with a limit.  If CTAs that want more than the
+// SM's 512 columns between them were resident together, two could wait for each other for good.  So a CTA asks for at least this
+// much shared memory: whatever fits an SM's 228 KB together (1 KB of which goes to each CTA) then wants 512 columns at most,
+// whatever the kernels' register counts.  All 512 columns: 228 - 181 KB leave no room for a second CTA; 256: two of them leave
+// 50 KB, one leaves room for two of 128; 128 or fewer: four.
+constexpr size_t least_smem(uint32_t columns) { return (columns > 256 ? 180 : columns > 128 ? 88 : 52) * 1024; }
+
 constexpr uint64_t kWaitLimitNs = 1000ull * 1000ull * 1000ull;   // 1 s per wait
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
