@@ -19,6 +19,8 @@
 // drains and frees its TMEM before it returns.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "gemm_epilogue.cuh"
 
 namespace glance {
@@ -657,48 +659,77 @@ bool tc_make_map_nd(CUtensorMap *map, const void *base, int n, const uint64_t *d
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// weight tiles of a launch (mode 1: 64 gate rows and their 64 up rows)
+static int tiles_of(int mode, int Nout) { return mode == 1 ? (Nout / 2 + 63) / 64 : (Nout + BM - 1) / BM; }
+
 // Equal row blocks: 144 rows are two blocks of 80 (padded), not 128 and 16.
 int tc_row_pad(int R) {
     const int blocks = (R + 127) / 128;
     return ((R + blocks - 1) / blocks + 15) / 16 * 16;
 }
 
-cudaError_t launch_gemm_tc(int mode, TcGemmArgs a, const CUtensorMap &map_w, const CUtensorMap &map_x, cudaStream_t st) {
-    a.np = tc_row_pad(a.R);
-    const int nb = a.x_lo_row > 0 ? 2 * a.np : a.np;
-    const int stage_bytes = BM * 128 + nb * 128;
+namespace {
+
+struct Ring {
+    int stages, stage_bytes;
+    uint32_t tmem_cols;
+    size_t smem;
+};
+
+// operand ring and tensor memory of a CTA of a launch of this shape
+Ring ring_of(int mode, int Nout, int R, int S, bool two_term) {
+    Ring r;
+    const int np = tc_row_pad(R), nb = two_term ? 2 * np : np;
+    r.stage_bytes = BM * 128 + nb * 128;
     // The ring stays under half of an SM's shared memory so that two CTAs fit per SM: a GPC then offers enough
     // CTA slots for every cluster of a launch to be resident in one wave, and one CTA's prologue and epilogue
     // overlap the other's streaming.
-    const int tiles = mode == 1 ? (a.F + 63) / 64 : (a.Nout + BM - 1) / BM;
+    const int tiles = tiles_of(mode, Nout);
     // The LM heads have a few more tiles than two CTAs per SM take in four rounds (1188 against 1184 at the 7B
     // vocabulary): with a smaller ring three CTAs fit per SM and the last round is as full as the others.
     const bool three = (mode == 0 || mode == 2 || mode == 5) && tiles > 3 * 148;
     // A launch of at most one CTA per SM takes a whole SM's ring: more of its weights, often all of them, are fetched before
     // the dependency wait (gate/up of 131 rows, h 1024, 88 CTAs: 13.6 -> 9.5 us).  With more CTAs the same ring would cost the
     // second CTA of an SM (down of the 7B widths, S 5: 23.5 -> 44 us).
-    const int row_blocks = (a.R + 127) / 128;
-    const bool alone = mode != 0 && !three && tiles * a.S * row_blocks <= 148;
-    int stages = (int)(((three ? 72 : alone ? 200 : 100) * 1024) / stage_bytes);
-    stages = stages > 12 ? 12 : (stages < 2 ? 2 : stages);
-    a.stages = stages;
-    uint32_t cols = 32;
-    while ((int)cols < nb) cols <<= 1;
-    a.tmem_cols = cols;
-    const size_t smem = (size_t)stages * stage_bytes + 1024;
+    const int row_blocks = (R + 127) / 128;
+    const bool alone = mode != 0 && !three && tiles * S * row_blocks <= 148;
+    r.stages = (int)(((three ? 72 : alone ? 200 : 100) * 1024) / r.stage_bytes);
+    r.stages = r.stages > 12 ? 12 : (r.stages < 2 ? 2 : r.stages);
+    r.tmem_cols = 32;
+    while ((int)r.tmem_cols < nb) r.tmem_cols <<= 1;
+    // Blocks of 65 to 80 rows with two terms have two slots of 36 KB and 256 columns: three such CTAs would fit an SM's shared
+    // memory, and the third waited in its allocation for one of the others (gate/up of 132 rows, h 2304, ffn 6144: 52 us; with
+    // two CTAs an SM 29)
+    r.smem = std::max((size_t)r.stages * r.stage_bytes + 1024, least_smem(r.tmem_cols));
+    return r;
+}
+
+}  // namespace
+
+CtaSize tc_cta_size(int mode, int Nout, int R, int S, bool two_term) {
+    const Ring r = ring_of(mode, Nout, R, S, two_term);
+    return CtaSize{(long long)r.smem, (long long)r.tmem_cols};
+}
+
+cudaError_t launch_gemm_tc(int mode, TcGemmArgs a, const CUtensorMap &map_w, const CUtensorMap &map_x, cudaStream_t st) {
+    const Ring r = ring_of(mode, a.Nout, a.R, a.S, a.x_lo_row > 0);
+    a.np = tc_row_pad(a.R);
+    a.stages = r.stages;
+    a.tmem_cols = r.tmem_cols;
+    const int tiles = tiles_of(mode, a.Nout), row_blocks = (a.R + 127) / 128;
     a.rows_fastest = row_blocks > 1 ? 1 : 0;
     dim3 grid(a.rows_fastest ? row_blocks : tiles, a.S, a.rows_fastest ? tiles : row_blocks);
     if (mode == 3 || mode == 4) {
         // every CTA's ring must hold S planes of ceil(np/S) rows, and a cluster has at most 8 CTAs
         const size_t rp = (a.np + a.S - 1) / a.S;
-        if (a.S > 8 || (size_t)a.S * rp * BM * 4 > (size_t)stages * stage_bytes) return cudaErrorInvalidValue;
+        if (a.S > 8 || (size_t)a.S * rp * BM * 4 > (size_t)r.stages * r.stage_bytes) return cudaErrorInvalidValue;
     }
-    if (mode == 0) return launch_mode<0>(a, map_w, map_x, smem, grid, st);
-    if (mode == 1) return launch_mode<1>(a, map_w, map_x, smem, grid, st);
-    if (mode == 2) return launch_mode<2>(a, map_w, map_x, smem, grid, st);
-    if (mode == 3) return launch_mode<3>(a, map_w, map_x, smem, grid, st);
-    if (mode == 5) return launch_mode<5>(a, map_w, map_x, smem, grid, st);
-    return launch_mode<4>(a, map_w, map_x, smem, grid, st);
+    if (mode == 0) return launch_mode<0>(a, map_w, map_x, r.smem, grid, st);
+    if (mode == 1) return launch_mode<1>(a, map_w, map_x, r.smem, grid, st);
+    if (mode == 2) return launch_mode<2>(a, map_w, map_x, r.smem, grid, st);
+    if (mode == 3) return launch_mode<3>(a, map_w, map_x, r.smem, grid, st);
+    if (mode == 5) return launch_mode<5>(a, map_w, map_x, r.smem, grid, st);
+    return launch_mode<4>(a, map_w, map_x, r.smem, grid, st);
 }
 
 }  // namespace glance

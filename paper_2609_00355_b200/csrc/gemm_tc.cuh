@@ -83,6 +83,7 @@ bool tc_make_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t ro
 bool tc_make_map_nd(CUtensorMap *map, const void *base, int n, const uint64_t *dims, const uint64_t *row_steps, const uint32_t *box);
 // activation rows per CTA, padded to the UMMA N granularity (box_rows of the X map)
 int tc_row_pad(int R);
+CtaSize tc_cta_size(int mode, int Nout, int R, int S, bool two_term);
 // mode: 0 fp32 planes, 1 SwiGLU, 2 arg-max, 3 cluster split-K + residual, 4 cluster split-K + rotary/KV write,
 // 5 per-tile top-k candidates + log-sum-exp shares.
 // map_w box_rows must be 128 (64 in mode 1), map_x box_rows tc_row_pad(R).
@@ -100,6 +101,7 @@ struct WideShape {
     long long steps;                 // 64-wide k-steps of the whole launch
 };
 WideShape wide_shape(int mode, int Nout, int K, int R);
+CtaSize wide_cta_size(int mode, int Nout, int K, int R, bool two_term);
 // map of W [Nout][K] for a mode of gemm_wide_kernel; the X map's box_rows is WideShape::np / 2
 bool wide_make_map(CUtensorMap *map, int mode, const void *W, int Nout, int K, int head_dim);
 // mode 1, 2, 3 or 4; S and the fields "filled by launch" are ignored

@@ -751,22 +751,44 @@ WideShape wide_shape(int mode, int Nout, int K, int R) {
     return s;
 }
 
+namespace {
+
+struct Ring {
+    int stages;
+    uint32_t tmem_cols;
+    size_t smem;
+};
+
+Ring ring_of(const WideShape &s, bool two_term) {
+    Ring r;
+    const int stage_bytes = BM * 128 + (two_term ? 2 : 1) * (s.np / 2) * 128;
+    r.stages = std::min(MAX_STAGES, (kWideSmem - 1024) / stage_bytes);
+    r.tmem_cols = 32;
+    while ((int)r.tmem_cols < 2 * s.np) r.tmem_cols <<= 1;
+    r.smem = std::max((size_t)r.stages * stage_bytes + 1024, least_smem(r.tmem_cols));
+    return r;
+}
+
+}  // namespace
+
+CtaSize wide_cta_size(int mode, int Nout, int K, int R, bool two_term) {
+    const Ring r = ring_of(wide_shape(mode, Nout, K, R), two_term);
+    return CtaSize{(long long)r.smem, (long long)r.tmem_cols};
+}
+
 cudaError_t launch_gemm_wide(int mode, TcGemmArgs a, const WideShape &s, const CUtensorMap &map_w, const CUtensorMap &map_x,
                              cudaStream_t st) {
     a.np = s.np;
     a.wide_pairs = s.pairs; a.wide_row_tiles = s.row_tiles; a.wide_rounds = s.rounds; a.wide_cut = s.cut; a.wide_items = s.items;
     a.wide_cutters = s.cutters;
-    const int stage_bytes = BM * 128 + (a.x_lo_row > 0 ? 2 : 1) * (s.np / 2) * 128;
-    a.stages = std::min(MAX_STAGES, (kWideSmem - 1024) / stage_bytes);
-    uint32_t cols = 32;
-    while ((int)cols < 2 * s.np) cols <<= 1;
-    a.tmem_cols = cols;
-    const size_t smem = (size_t)a.stages * stage_bytes + 1024;
+    const Ring r = ring_of(s, a.x_lo_row > 0);
+    a.stages = r.stages;
+    a.tmem_cols = r.tmem_cols;
     if (s.cut > kWideCut || s.pairs > kWidePairs || s.np > kWideRows) return cudaErrorInvalidValue;
-    if (mode == 1) return launch_mode<1>(a, map_w, map_x, smem, st);
-    if (mode == 2) return launch_mode<2>(a, map_w, map_x, smem, st);
-    if (mode == 3) return launch_mode<3>(a, map_w, map_x, smem, st);
-    return launch_mode<4>(a, map_w, map_x, smem, st);
+    if (mode == 1) return launch_mode<1>(a, map_w, map_x, r.smem, st);
+    if (mode == 2) return launch_mode<2>(a, map_w, map_x, r.smem, st);
+    if (mode == 3) return launch_mode<3>(a, map_w, map_x, r.smem, st);
+    return launch_mode<4>(a, map_w, map_x, r.smem, st);
 }
 
 }  // namespace glance

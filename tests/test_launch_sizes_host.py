@@ -26,6 +26,22 @@ def _attention_sizes(lib):
     return [fn(d) for d in (64, 128)]
 
 
+def _gemm_sizes(lib):
+    tc = lib._ZN6glance11tc_cta_sizeEiiiib
+    tc.restype, tc.argtypes = CtaSize, [C.c_int] * 4 + [C.c_bool]
+    wide = lib._ZN6glance13wide_cta_sizeEiiiib
+    wide.restype, wide.argtypes = CtaSize, [C.c_int] * 4 + [C.c_bool]
+    out = []
+    for R in list(range(1, 129)) + [129, 144, 160, 161, 257, 577, 1280]:
+        for mode, two in ((0, False), (1, True), (1, False), (2, False), (3, True), (4, False), (5, False)):
+            for Nout in (256, 4608, 37888, 152064):
+                for S in (1, 2, 8) if mode in (3, 4) else (1,):
+                    out.append(tc(mode, Nout, R, S, two))
+        if R > 128:
+            out += [wide(mode, 8192, 4096, R, mode in (1, 3)) for mode in (1, 2, 3, 4)]
+    return out
+
+
 def _most_columns(sizes):
     """The most columns that CTAs which fit an SM's shared memory together can want."""
     items = sorted({(s.smem + PER_CTA, s.columns) for s in sizes})
@@ -40,6 +56,6 @@ def _most_columns(sizes):
 def test_ctas_that_fit_an_sm_fit_its_tensor_memory(lib):
     """A CTA that waits for columns, held by one that waits for it, would wait for good: shared memory alone has to keep such
     CTAs apart (the kernels' register counts do not count here)."""
-    sizes = _attention_sizes(lib)
+    sizes = _attention_sizes(lib) + _gemm_sizes(lib)
     assert all(0 < s.smem <= 227 * 1024 and s.columns <= SM_COLUMNS for s in sizes)
     assert _most_columns(sizes) <= SM_COLUMNS
