@@ -20,6 +20,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "gemm_epilogue.cuh"
 
@@ -668,6 +669,74 @@ int tc_row_pad(int R) {
     return ((R + blocks - 1) / blocks + 15) / 16 * 16;
 }
 
+// Clusters of `size` CTAs with a whole SM's ring each (modes 3 and 4) that are resident at once: a cluster starts when one GPC
+// has that many SMs free.  148 / 74 / 45 / 33 / 26 / 22 / 15 / 15 of one to eight CTAs, which is also the answer where there is
+// no device to ask.
+int tc_resident_clusters(int size) {
+    static const int known[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+    static int cache[9] = {0};
+    if (size < 1 || size > 8) return 0;
+    if (cache[size] == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1, size, 1);
+        cfg.blockDim = dim3(NTHR, 1, 1);
+        cfg.dynamicSmemBytes = 200 * 1024;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1;
+        attr[0].val.clusterDim.y = size;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaFuncSetAttribute(gemm_tc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, gemm_tc_kernel<3>, &cfg) != cudaSuccess || n < 1) {
+            (void)cudaGetLastError();
+            n = known[size];
+        }
+        cache[size] = n;
+    }
+    return cache[size];
+}
+
+// Split-K factor of a weight-streaming GEMM.  The splits of one tile form a thread-block cluster (<= 8 CTAs) that reduces them
+// through shared memory.  Up to 128 rows: as many CTAs as fit one wave at two CTAs per SM (one CTA per SM with half a ring
+// keeps too few weight bytes in flight to cover the HBM latency) with at least 7 k-tiles each, and more and shorter ones where
+// even those leave SMs idle.  More row blocks: by the time of a k-step, the exchange at the end and the waves.
+int tc_splits(int Nout, int K, int rows, bool two_term) {
+    const int tiles = (Nout + 127) / 128;
+    const int ktiles = K / 64;
+    const int row_blocks = (rows + 127) / 128;
+    if (row_blocks > 1) {
+        // A k-step of a CTA is bound by the arrival of its operands, and the exchange at the end costs about the same
+        // whatever the split (us, one 7B layer: QKV at 144 rows S = 1 / 2 / 3 / 4: 35 / 22 / 18 / 29, O 45 / 27 / 21 / 18 and 26
+        // with five; 256 rows: QKV 43 / 27 / 23 / 35, O 54 / 32 / 25 / 22 and 30).  The jumps are launches that no longer fit
+        // at once: 296 CTAs are resident without clusters or in pairs, about 250 in larger clusters -- which a long loop makes up
+        // for (down, 56 tiles and blocks, four and five splits: 59 / 53 at 144 rows, 79 / 61 at 256).
+        const double step_us = 0.29 + 0.002 * tc_row_pad(rows) * (two_term ? 2 : 1);
+        const int smax = std::max(1, std::min(8, ktiles / 2));
+        int best = 1;
+        double best_us = 1e30;
+        for (int s = 1; s <= smax; ++s) {
+            const double waves = std::ceil((double)tiles * row_blocks * s / (s <= 2 || ktiles >= 40 * s ? 296.0 : 250.0));
+            const double us = waves * (ktiles * step_us / s + 9.5);
+            if (us < best_us - 1e-9) { best_us = us; best = s; }
+        }
+        return best;
+    }
+    int s = (2 * 148) / tiles;
+    s = std::min(s, std::max(1, ktiles / 7));
+    s = std::max(1, std::min(s, 8));
+    // A launch of few CTAs: more and shorter splits, whose weights are all fetched before the predecessor is done (small model,
+    // h 1024, 32 rows, QKV / O / down: 7.5 / 7.5 / 7.4 us with 2 / 2 / 6 splits, 6.4 / 5.3 / 6.8 with eight and whole rings) --
+    // as far as their clusters are resident at one CTA per SM.  Layers at 16 rows: h 2304 65.5 us with eight splits that were
+    // not, 54.1 now; 2048 (ffn 11008) 77.0 -> 59.4; 1792 52.1 -> 47.5.
+    for (int f = std::min(8, ktiles / 2); f > s; --f)
+        if (tiles <= tc_resident_clusters(f)) s = f;
+    if (s == 8 && tiles > 33) s = 7;                   // at most 33 clusters of eight are resident at two CTAs per SM
+    return s;
+}
+
 namespace {
 
 struct Ring {
@@ -688,11 +757,12 @@ Ring ring_of(int mode, int Nout, int R, int S, bool two_term) {
     // The LM heads have a few more tiles than two CTAs per SM take in four rounds (1188 against 1184 at the 7B
     // vocabulary): with a smaller ring three CTAs fit per SM and the last round is as full as the others.
     const bool three = (mode == 0 || mode == 2 || mode == 5) && tiles > 3 * 148;
-    // A launch of at most one CTA per SM takes a whole SM's ring: more of its weights, often all of them, are fetched before
-    // the dependency wait (gate/up of 131 rows, h 1024, 88 CTAs: 13.6 -> 9.5 us).  With more CTAs the same ring would cost the
-    // second CTA of an SM (down of the 7B widths, S 5: 23.5 -> 44 us).
+    // A launch that is resident at one CTA per SM takes a whole SM's ring: more of its weights, often all of them, are fetched
+    // before the dependency wait (gate/up of 131 rows, h 1024, 88 CTAs: 13.6 -> 9.5 us).  With more CTAs the same ring would
+    // cost the second CTA of an SM (down of the 7B widths, S 5: 23.5 -> 44 us), and with more clusters than the GPCs hold a
+    // second wave (h 2304, 16 rows, O of 18 clusters of eight: 7.0 -> 13.5 us).
     const int row_blocks = (R + 127) / 128;
-    const bool alone = mode != 0 && !three && tiles * S * row_blocks <= 148;
+    const bool alone = mode != 0 && !three && tiles * row_blocks <= (mode == 3 || mode == 4 ? tc_resident_clusters(S) : 148);
     r.stages = (int)(((three ? 72 : alone ? 200 : 100) * 1024) / r.stage_bytes);
     r.stages = r.stages > 12 ? 12 : (r.stages < 2 ? 2 : r.stages);
     r.tmem_cols = 32;

@@ -83,6 +83,9 @@ bool tc_make_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t ro
 bool tc_make_map_nd(CUtensorMap *map, const void *base, int n, const uint64_t *dims, const uint64_t *row_steps, const uint32_t *box);
 // activation rows per CTA, padded to the UMMA N granularity (box_rows of the X map)
 int tc_row_pad(int R);
+int tc_resident_clusters(int size);
+// split-K factor of modes 3 and 4: K splits of one tile, a thread-block cluster
+int tc_splits(int Nout, int K, int rows, bool two_term);
 CtaSize tc_cta_size(int mode, int Nout, int R, int S, bool two_term);
 // mode: 0 fp32 planes, 1 SwiGLU, 2 arg-max, 3 cluster split-K + residual, 4 cluster split-K + rotary/KV write,
 // 5 per-tile top-k candidates + log-sum-exp shares.

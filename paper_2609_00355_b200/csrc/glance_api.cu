@@ -16,43 +16,6 @@ namespace {
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// split-K factor of a weight-streaming GEMM: as many CTAs as fit one wave at two CTAs per SM (one CTA per SM
-// keeps too few weight bytes in flight to cover the HBM latency), at least 7 k-tiles per split
-// The splits of one tile form a thread-block cluster (<= 8 CTAs) that reduces them through shared memory.
-// With more than one 128-row block the launch is tensor-bound, not latency-bound: every (tile, row block) item is a
-// long main loop, and splitting K only pays where it evens out the last wave over the 148 SMs -- each split adds a
-// cluster epilogue of a few microseconds per item.
-int choose_split(int Nout, int K, int rows, bool two_term) {
-    const int tiles = (Nout + 127) / 128;
-    const int ktiles = K / 64;
-    const int row_blocks = (rows + 127) / 128;
-    if (row_blocks > 1) {
-        // A k-step of a CTA is bound by the arrival of its operands, and the exchange at the end costs about the same
-        // whatever the split (us, one 7B layer: QKV at 144 rows S = 1 / 2 / 3 / 4: 35 / 22 / 18 / 29, O 45 / 27 / 21 / 18 and 26
-        // with five; 256 rows: QKV 43 / 27 / 23 / 35, O 54 / 32 / 25 / 22 and 30).  The jumps are launches that no longer fit
-        // at once: 296 CTAs are resident without clusters or in pairs, about 250 in larger clusters -- which a long loop makes up
-        // for (down, 56 tiles and blocks, four and five splits: 59 / 53 at 144 rows, 79 / 61 at 256).
-        const double step_us = 0.29 + 0.002 * tc_row_pad(rows) * (two_term ? 2 : 1);
-        const int smax = std::max(1, std::min(8, ktiles / 2));
-        int best = 1;
-        double best_us = 1e30;
-        for (int s = 1; s <= smax; ++s) {
-            const double waves = std::ceil((double)tiles * row_blocks * s / (s <= 2 || ktiles >= 40 * s ? 296.0 : 250.0));
-            const double us = waves * (ktiles * step_us / s + 9.5);
-            if (us < best_us - 1e-9) { best_us = us; best = s; }
-        }
-        return best;
-    }
-    int s = (2 * 148) / tiles;
-    s = std::min(s, std::max(1, ktiles / 7));
-    // a launch of few CTAs: more and shorter splits, whose weights are all fetched before the predecessor is done (small model,
-    // h 1024, 32 rows, QKV / O / down: 7.5 / 7.5 / 7.4 us with 2 / 2 / 6 splits, 6.4 / 5.3 / 6.8 with eight and whole rings)
-    s = std::max(s, std::min(148 / tiles, ktiles / 2));
-    s = std::max(1, std::min(s, 8));
-    if (s == 8 && tiles > 33) s = 7;                   // at most 33 clusters of eight are resident at two CTAs per SM
-    return s;
-}
-
 // Rows of one prefill pass (bounded by the sequence's capacity).  Every pass reads all weights, so a pass of N rows
 // costs their 14 GB at the 7B widths whatever N is, until the tensor work of the rows is as long (about 300 rows with
 // two-term activations).  At 2048 rows the weights are 10 % of the pass and the activations take 0.3 GB of workspace.
@@ -383,7 +346,7 @@ void run_layer(glance_ctx *ctx, const LayerW &w, bf16 *pool_layer, const PassInf
     const int xr = d.Rmax;                             // rows allocated behind every activation buffer
     {
         TcGemmArgs g{};
-        g.Nout = d.qkv_out; g.K = c.hidden; g.R = ps.R; g.S = choose_split(d.qkv_out, c.hidden, ps.R, false);
+        g.Nout = d.qkv_out; g.K = c.hidden; g.R = ps.R; g.S = tc_splits(d.qkv_out, c.hidden, ps.R, false);
         with_row_scales(ctx, g);
         g.x_lo_row = 0;      // q, K, V are rounded to bf16 right after: the second term of x would buy nothing
         g.q = ws.q; g.q_lo = ws.q + (size_t)xr * d.qd; g.pool_layer = pool_layer; g.kvrow = ws.row_kvrow;
@@ -393,7 +356,7 @@ void run_layer(glance_ctx *ctx, const LayerW &w, bf16 *pool_layer, const PassInf
         const bf16 *wqkv = w.wqkv;
         if (ps.Rq == 0) {     // no row continues as a query (prefill of the head's context): the K and V features only
             wqkv += (size_t)d.qd * c.hidden;
-            g.Nout = d.qkv_out - d.qd; g.Hq = 0; g.S = choose_split(g.Nout, c.hidden, ps.R, false);
+            g.Nout = d.qkv_out - d.qd; g.Hq = 0; g.S = tc_splits(g.Nout, c.hidden, ps.R, false);
         }
         gemm(ctx, 4, wqkv, ws.xn, xr, g);
     }
@@ -409,7 +372,7 @@ void run_layer(glance_ctx *ctx, const LayerW &w, bf16 *pool_layer, const PassInf
     const int R = ps.Rq;
     {
         TcGemmArgs g{};
-        g.Nout = c.hidden; g.K = d.qd; g.R = R; g.S = choose_split(c.hidden, d.qd, R, true);
+        g.Nout = c.hidden; g.K = d.qd; g.R = R; g.S = tc_splits(c.hidden, d.qd, R, true);
         g.x = ws.x; g.gain = w.ln2; g.xb = ws.xn; g.xb_lo = ws.xn + (size_t)xr * c.hidden; g.ssq_out = ws.ssq;
         g.ssq_stride = d.Rmax; g.x_lo_row = xr;
         gemm(ctx, 3, w.wo, ws.attn, xr, g);
@@ -423,7 +386,7 @@ void run_layer(glance_ctx *ctx, const LayerW &w, bf16 *pool_layer, const PassInf
     }
     {
         TcGemmArgs g{};
-        g.Nout = c.hidden; g.K = c.ffn; g.R = R; g.S = choose_split(c.hidden, c.ffn, R, true);
+        g.Nout = c.hidden; g.K = c.ffn; g.R = R; g.S = tc_splits(c.hidden, c.ffn, R, true);
         g.x = ws.x; g.gain = next_gain; g.xb = ws.xn; g.xb_lo = ws.xn + (size_t)xr * c.hidden; g.hidden_out = hidden_out;
         g.ssq_out = ws.ssq; g.ssq_stride = d.Rmax; g.x_lo_row = xr;
         gemm(ctx, 3, w.wd, ws.act, xr, g);

@@ -59,3 +59,27 @@ def test_ctas_that_fit_an_sm_fit_its_tensor_memory(lib):
     sizes = _attention_sizes(lib) + _gemm_sizes(lib)
     assert all(0 < s.smem <= 227 * 1024 and s.columns <= SM_COLUMNS for s in sizes)
     assert _most_columns(sizes) <= SM_COLUMNS
+
+
+RESIDENT = {1: 148, 2: 74, 3: 45, 4: 33, 5: 26, 6: 22, 7: 15, 8: 15}     # clusters of a size at one CTA per SM
+
+
+@pytest.mark.parametrize("two_term", [False, True])
+def test_launches_with_a_whole_sm_to_a_cta_are_resident_at_once(lib, two_term):
+    """A ring that takes an SM for itself must not leave clusters of the launch to a second wave, and the planes of a cluster's
+    splits fit the ring."""
+    splits = lib._ZN6glance9tc_splitsEiiib
+    splits.restype, splits.argtypes = C.c_int, [C.c_int] * 3 + [C.c_bool]
+    size = lib._ZN6glance11tc_cta_sizeEiiiib
+    size.restype, size.argtypes = CtaSize, [C.c_int] * 4 + [C.c_bool]
+    for tiles in range(1, 80):
+        for ktiles in (1, 2, 8, 20, 36, 96, 296):
+            for R in (1, 16, 32, 65, 96, 128, 132, 192, 320, 600, 1100):
+                S = splits(128 * tiles, 64 * ktiles, R, two_term)
+                blocks = -(-R // 128)
+                rows = -(-(-(-R // blocks)) // 16) * 16
+                s = size(3 if two_term else 4, 128 * tiles, R, S, two_term)
+                assert 1 <= S <= min(8, ktiles)
+                assert S * -(-rows // S) * 512 <= s.smem - 1024
+                if 2 * (s.smem + PER_CTA) > SM_SMEM:
+                    assert tiles * blocks <= RESIDENT[S], (tiles, ktiles, R, S)
