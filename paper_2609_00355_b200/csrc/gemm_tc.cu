@@ -711,15 +711,18 @@ int tc_splits(int Nout, int K, int rows, bool two_term) {
         // A k-step of a CTA is bound by the arrival of its operands, and the exchange at the end costs about the same
         // whatever the split (us, one 7B layer: QKV at 144 rows S = 1 / 2 / 3 / 4: 35 / 22 / 18 / 29, O 45 / 27 / 21 / 18 and 26
         // with five; 256 rows: QKV 43 / 27 / 23 / 35, O 54 / 32 / 25 / 22 and 30).  The jumps are launches that no longer fit
-        // at once: 296 CTAs are resident without clusters or in pairs, about 250 in larger clusters -- which a long loop makes up
-        // for (down, 56 tiles and blocks, four and five splits: 59 / 53 at 144 rows, 79 / 61 at 256).
+        // at once: 296 CTAs are resident without clusters or in pairs, and of larger clusters twice what is resident at one CTA
+        // per SM (66 clusters of four fit, 72 don't; 90 of three fit) -- which a long loop makes up for (down, 56 tiles and
+        // blocks, four and five splits: 59 / 53 at 144 rows, 79 / 61 at 256).
         const double step_us = 0.29 + 0.002 * tc_row_pad(rows) * (two_term ? 2 : 1);
         const int smax = std::max(1, std::min(8, ktiles / 2));
         int best = 1;
         double best_us = 1e30;
         for (int s = 1; s <= smax; ++s) {
-            const double waves = std::ceil((double)tiles * row_blocks * s / (s <= 2 || ktiles >= 40 * s ? 296.0 : 250.0));
-            const double us = waves * (ktiles * step_us / s + 9.5);
+            const int at_once = s <= 2 || ktiles >= 40 * s ? 296 / s : std::max(2 * tc_resident_clusters(s), 250 / s);
+            const double waves = std::ceil((double)tiles * row_blocks / at_once);
+            // clusters of a later wave also wait for SMs of one GPC to come free together
+            const double us = waves * (ktiles * step_us / s + 9.5) + (waves > 1.0 && s > 2 ? 3.0 : 0.0);
             if (us < best_us - 1e-9) { best_us = us; best = s; }
         }
         return best;

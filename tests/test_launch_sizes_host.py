@@ -83,3 +83,12 @@ def test_launches_with_a_whole_sm_to_a_cta_are_resident_at_once(lib, two_term):
                 assert S * -(-rows // S) * 512 <= s.smem - 1024
                 if 2 * (s.smem + PER_CTA) > SM_SMEM:
                     assert tiles * blocks <= RESIDENT[S], (tiles, ktiles, R, S)
+
+
+@pytest.mark.parametrize("hidden,K,rows,S", [(2816, 7680, 384, 4), (1792, 4864, 768, 3), (2816, 2816, 512, 3), (3328, 8960, 256, 5),
+                                             (3584, 3584, 144, 4), (2304, 2304, 1280, 1)])
+def test_split_factors_use_the_clusters_that_fit_at_two_ctas_an_sm(lib, hidden, K, rows, S):
+    """66 clusters of four and 84 of three are one wave; 180 of three would be two full ones for an unsplit one."""
+    splits = lib._ZN6glance9tc_splitsEiiib
+    splits.restype, splits.argtypes = C.c_int, [C.c_int] * 3 + [C.c_bool]
+    assert splits(hidden, K, rows, True) == S
