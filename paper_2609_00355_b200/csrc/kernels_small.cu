@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(32) topk_stage2_kernel(int k, int n_warps, con
 // entries reach it), or of a warp's lane maxima where it has fewer than k warps; the few keys that reach it (about 12 of
 // 19000) are ranked by counting the larger ones.  15 rows of 152064, k 8: 18.4 us a call with the two launches (13.8 on the
 // device, the second being 15 single warps over 1192 keys each), 14.7 with this one.  A cluster of eight holds 192 spans in
-// registers; longer rows take the two launches.
+// registers; longer rows, and more rows than clusters are resident (topk_one_launch()), take the two launches.
 // ------------------------------------------------------------------------------------------
 constexpr int kRowWarps = 24;                            // warps of a CTA at most
 constexpr int kRowCluster = 8;
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) topk_row_kernel(const float *l
                                                                   int32_t *ids, float *lp) {
     // Keys a CTA collects before it falls back to exact selection.  About 30 where the bound is one of its warps' maxima, but
     // 22 a warp where it is the 16th largest lane maximum of one (k 16, fewer than 16 warps): with 128 places those fell back
-    // (15 rows of 65000, k 16: 27.7 us, now 10.1).
+    // (15 rows of 65000, k 16: 27.7 us, now 10.2).
     constexpr int CAP = 512;
     __shared__ uint32_t bound[2][kRowWarps];
     __shared__ unsigned long long list[CAP], best[kMaxTopk], warp_best[kRowWarps];
@@ -534,23 +534,58 @@ __global__ void __launch_bounds__(kRowWarps * 32) topk_row_kernel(const float *l
 
 int topk_warps(int V) { return (V + kTopkWarpSpan - 1) / kTopkWarpSpan; }
 
+// The one launch is chosen where a row's cluster need not wait for another's to end: a CTA of a long row has an SM to itself
+// (80 registers, 13 warps and more), so 15 clusters are resident, and what they do after their loads overlaps with nothing.
+// With k of 8 and more, and rows of at least 32 spans, the second launch's single warps cost more than a second round.  us,
+// two launches / one: V 152064, 15 rows, k 8: 14.3 / 7.7; 30 rows, k 8 20.5 / 15.6, k 4 16.8 / 15.7, k 1 12.9 / 13.8; 60 rows,
+// k 4 22.0 / 25.4; 90 rows, k 8 36.5 / 39.0; V 8193, 120 rows, k 4 8.9 / 7.3, 150 rows (142 are resident) 9.1 / 10.6.
+bool topk_one_launch(int rows, int spans, int k, int resident) {
+    return rows <= resident || (rows <= 2 * resident && spans >= 32 && k >= 8);
+}
+
+namespace {
+
+cudaLaunchConfig_t row_config(int ctas, int warps, int rows, cudaStream_t st, cudaLaunchAttribute *attr) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas, rows, 1);
+    cfg.blockDim = dim3(32 * warps, 1, 1);
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// rows whose clusters are resident at once (asked once per shape)
+int resident_rows(int ctas, int warps) {
+    static int cache[2][kRowWarps + 1] = {{0}};
+    int &n = cache[ctas > 1 ? 1 : 0][warps];
+    if (n == 0) {
+        cudaLaunchAttribute attr[1];
+        const cudaLaunchConfig_t cfg = row_config(ctas, warps, 1, nullptr, attr);
+        int got = 0;
+        if (cudaOccupancyMaxActiveClusters(&got, topk_row_kernel, &cfg) != cudaSuccess || got < 1) {
+            (void)cudaGetLastError();
+            got = ctas > 1 ? 15 : 148;
+        }
+        n = got;
+    }
+    return n;
+}
+
+}  // namespace
+
 void launch_topk(const float *logits, int batch, int B, int V, int k, int32_t *ids, float *lp,
                  unsigned long long *cand, float *ml, cudaStream_t st) {
     if (B < 2) return;
     const int rows = batch * (B - 1), nw = topk_warps(V);
-    if (nw <= kRowSpans) {
-        const int ctas = nw > 8 ? kRowCluster : 1;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(ctas, rows, 1);
-        cfg.blockDim = dim3(32 * ((nw + ctas - 1) / ctas), 1, 1);
-        cfg.stream = st;
+    const int ctas = nw > 8 ? kRowCluster : 1, warps = (nw + ctas - 1) / ctas;
+    if (nw <= kRowSpans && topk_one_launch(rows, nw, k, resident_rows(ctas, warps))) {
         cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = ctas;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        const cudaLaunchConfig_t cfg = row_config(ctas, warps, rows, st, attr);
         cudaLaunchKernelEx(&cfg, topk_row_kernel, logits, B, V, k, nw, ids, lp);
         return;
     }

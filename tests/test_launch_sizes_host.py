@@ -92,3 +92,12 @@ def test_split_factors_use_the_clusters_that_fit_at_two_ctas_an_sm(lib, hidden, 
     splits = lib._ZN6glance9tc_splitsEiiib
     splits.restype, splits.argtypes = C.c_int, [C.c_int] * 3 + [C.c_bool]
     assert splits(hidden, K, rows, True) == S
+
+
+@pytest.mark.parametrize("rows,spans,k,resident,one", [(15, 149, 1, 15, True), (16, 149, 7, 15, False), (30, 149, 8, 15, True),
+                                                       (31, 149, 16, 15, False), (142, 9, 1, 142, True), (143, 9, 16, 142, False),
+                                                       (48, 64, 1, 48, True), (60, 64, 4, 48, False), (3000, 8, 4, 444, False)])
+def test_topk_takes_one_launch_while_its_clusters_are_resident(lib, rows, spans, k, resident, one):
+    fn = lib._ZN6glance15topk_one_launchEiiii
+    fn.restype, fn.argtypes = C.c_bool, [C.c_int] * 4
+    assert fn(rows, spans, k, resident) is one

@@ -109,3 +109,22 @@ def test_topk_static_edges_of_spans_and_lists(V, k, kind):
         assert np.array_equal(np.isfinite(got), fin)
         # fp32 sums of V terms in blocks of 32 and more: 1e-6 of the log-sum-exp's scale
         assert np.abs(got[fin] - ref[fin]).max() <= 4e-6 * max(1.0, float(np.abs(row[np.isfinite(row)]).max()) + np.log(V))
+
+
+@pytest.mark.parametrize("batch,B,V,k", [(2, 16, 152064, 8), (2, 16, 152064, 4), (4, 16, 152064, 4), (10, 16, 8193, 16), (32, 16, 8192, 4),
+                                         (1, 16, 65000, 16), (6, 16, 65000, 16), (2, 16, 8192, 16)])
+def test_topk_static_many_rows(batch, B, V, k):
+    """More rows than clusters are resident, in one launch and in two, and lists of more than 128 keys, against the exact
+    (logit desc, id asc) order; the log-probabilities against 64 bits (fp32 sums of V terms: 1e-6 of the scale)."""
+    from paper_2609_00355_b200 import binding
+    g = torch.Generator(device="cuda").manual_seed(V + k)
+    x = torch.randn(batch, B, V, generator=g, device="cuda") * 1.2
+    ids = torch.full((batch, B - 1, k), -1, dtype=torch.int32, device="cuda")
+    lp = torch.full((batch, B - 1, k), float("nan"), dtype=torch.float32, device="cuda")
+    for _ in range(2):
+        assert binding.glance_topk_static(x, k, ids, lp) == 0
+    rows = x[:, 1:]
+    val, idx = torch.sort(rows, dim=-1, descending=True, stable=True)
+    assert torch.equal(ids.long(), idx[..., :k])
+    ref = val[..., :k].double() - torch.logsumexp(rows.double(), dim=-1, keepdim=True)
+    assert float((lp.double() - ref).abs().max()) <= 4e-6 * (float(rows.abs().max()) + np.log(V))
