@@ -67,7 +67,7 @@ void launch_setup_draft(const DraftSetup &p, cudaStream_t st);
 // rows (s, j), j = 1..L of logits [batch*B][V] -> ids/lp [batch][L][k]; scratch: cand [rows][topk_warps(V)][k],
 // ml [rows][topk_warps(V)][2].  One launch, which leaves the scratch alone, or two.
 int topk_warps(int V);
-bool topk_one_launch(int rows, int spans, int k, int resident);
+bool topk_one_launch(int rows, int spans, int warps, int k, int resident);
 void launch_topk(const float *logits, int batch, int B, int V, int k, int32_t *ids, float *lp,
                  unsigned long long *cand, float *ml, cudaStream_t st);
 

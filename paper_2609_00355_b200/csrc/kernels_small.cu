@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(32) topk_stage2_kernel(int k, int n_warps, con
 // entries reach it), or of a warp's lane maxima where it has fewer than k warps; the few keys that reach it (about 12 of
 // 19000) are ranked by counting the larger ones.  15 rows of 152064, k 8: 18.4 us a call with the two launches (13.8 on the
 // device, the second being 15 single warps over 1192 keys each), 14.7 with this one.  A cluster of eight holds 192 spans in
-// registers; longer rows, and more rows than clusters are resident (topk_one_launch()), take the two launches.
+// registers; longer rows, and more rows than clusters are resident for (topk_one_launch()), take the two launches.
 // ------------------------------------------------------------------------------------------
 constexpr int kRowWarps = 24;                            // warps of a CTA at most
 constexpr int kRowCluster = 8;
@@ -534,13 +534,17 @@ __global__ void __launch_bounds__(kRowWarps * 32) topk_row_kernel(const float *l
 
 int topk_warps(int V) { return (V + kTopkWarpSpan - 1) / kTopkWarpSpan; }
 
-// The one launch is chosen where a row's cluster need not wait for another's to end: a CTA of a long row has an SM to itself
-// (80 registers, 13 warps and more), so 15 clusters are resident, and what they do after their loads overlaps with nothing.
-// With k of 8 and more, and rows of at least 32 spans, the second launch's single warps cost more than a second round.  us,
-// two launches / one: V 152064, 15 rows, k 8: 14.3 / 7.7; 30 rows, k 8 20.5 / 15.6, k 4 16.8 / 15.7, k 1 12.9 / 13.8; 60 rows,
-// k 4 22.0 / 25.4; 90 rows, k 8 36.5 / 39.0; V 8193, 120 rows, k 4 8.9 / 7.3, 150 rows (142 are resident) 9.1 / 10.6.
-bool topk_one_launch(int rows, int spans, int k, int resident) {
-    return rows <= resident || (rows <= 2 * resident && spans >= 32 && k >= 8);
+// The one launch is chosen while every row's cluster is resident (a CTA of a long row has an SM to itself -- 80 registers, 13
+// warps and more -- which leaves 15 clusters), and beyond that as far as the second of two launches costs more than a further
+// round: its single warps go through k keys of every span, a round's loads and ranking overlap with nothing.  Rows of 9 to 31
+// spans are over too fast for a second round, and with more than eight warps, but fewer than k, a round ranks long lists.  us,
+// two launches / one: V 152064, 15 rows, k 8: 14.3 / 7.7; 45 rows, k 8 24.9 / 21.6, k 4 19.0 / 20.1, k 1 15.8 / 19.2; 60 rows,
+// k 4 22.0 / 25.4; 90 rows, k 8 36.5 / 39.0; V 65000 (48 resident), 90 rows, k 4 16.6 / 14.5; V 8193, 120 rows, k 4 8.9 / 7.3,
+// 150 rows (142 are resident) 9.1 / 10.6; V 100000, 45 rows, k 16 28.6 / 32.5.  `warps`: of a CTA.
+bool topk_one_launch(int rows, int spans, int warps, int k, int resident) {
+    if (rows <= resident) return true;
+    if ((spans > 8 && spans < 32) || (k > warps && warps > 8)) return false;
+    return 250ll * (rows - resident) <= (long long)resident * (k - 1) * spans;
 }
 
 namespace {
@@ -583,7 +587,7 @@ void launch_topk(const float *logits, int batch, int B, int V, int k, int32_t *i
     if (B < 2) return;
     const int rows = batch * (B - 1), nw = topk_warps(V);
     const int ctas = nw > 8 ? kRowCluster : 1, warps = (nw + ctas - 1) / ctas;
-    if (nw <= kRowSpans && topk_one_launch(rows, nw, k, resident_rows(ctas, warps))) {
+    if (nw <= kRowSpans && topk_one_launch(rows, nw, warps, k, resident_rows(ctas, warps))) {
         cudaLaunchAttribute attr[1];
         const cudaLaunchConfig_t cfg = row_config(ctas, warps, rows, st, attr);
         cudaLaunchKernelEx(&cfg, topk_row_kernel, logits, B, V, k, nw, ids, lp);

@@ -94,10 +94,11 @@ def test_split_factors_use_the_clusters_that_fit_at_two_ctas_an_sm(lib, hidden, 
     assert splits(hidden, K, rows, True) == S
 
 
-@pytest.mark.parametrize("rows,spans,k,resident,one", [(15, 149, 1, 15, True), (16, 149, 7, 15, False), (30, 149, 8, 15, True),
-                                                       (31, 149, 16, 15, False), (142, 9, 1, 142, True), (143, 9, 16, 142, False),
-                                                       (48, 64, 1, 48, True), (60, 64, 4, 48, False), (3000, 8, 4, 444, False)])
-def test_topk_takes_one_launch_while_its_clusters_are_resident(lib, rows, spans, k, resident, one):
-    fn = lib._ZN6glance15topk_one_launchEiiii
-    fn.restype, fn.argtypes = C.c_bool, [C.c_int] * 4
-    assert fn(rows, spans, k, resident) is one
+@pytest.mark.parametrize("rows,spans,warps,k,resident,one", [
+    (15, 149, 19, 1, 15, True), (16, 149, 19, 1, 15, False), (45, 149, 19, 8, 15, True), (60, 149, 19, 4, 15, False),
+    (98, 149, 19, 8, 15, False), (142, 9, 2, 1, 142, True), (143, 9, 2, 16, 142, False), (90, 64, 8, 4, 48, False),
+    (80, 64, 8, 4, 48, True), (16, 98, 13, 16, 15, False), (480, 8, 8, 4, 444, True), (3000, 8, 8, 16, 444, False)])
+def test_topk_takes_one_launch_while_its_clusters_are_resident(lib, rows, spans, warps, k, resident, one):
+    fn = lib._ZN6glance15topk_one_launchEiiiii
+    fn.restype, fn.argtypes = C.c_bool, [C.c_int] * 5
+    assert fn(rows, spans, warps, k, resident) is one
