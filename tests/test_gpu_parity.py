@@ -158,9 +158,10 @@ def _wide_operands(mode, Nout, K, R, terms):
     (1, 1408, 2304, 200, 2), (1, 20480, 256, 130, 2), (1, 128, 64, 129, 1), (1, 4096, 1024, 1000, 2),
     (2, 19000, 320, 129, 1), (2, 1000, 2304, 600, 1), (2, 255, 64, 300, 1), (2, 18945, 1024, 256, 1),
     (3, 2304, 8192, 144, 2), (3, 2112, 4096, 1024, 2), (3, 64, 64, 129, 1), (3, 192, 2304, 300, 2),
-    # shared items handed over by groups of rows: more and fewer parts than steps of 32 rows, rows that end inside a group;
-    # 66 items, a rest that is dealt out whole
-    (3, 512, 8192, 129, 2), (3, 1024, 8192, 250, 2), (2, 512, 8192, 161, 1), (1, 8448, 1024, 300, 2)])
+    # items in many parts, partial row tiles; a rest that is dealt out whole: 66 items, and 140, where some pairs stop an item
+    # earlier than the others, with both accumulators in use
+    (3, 512, 8192, 129, 2), (3, 1024, 8192, 250, 2), (2, 512, 8192, 161, 1), (1, 8448, 1024, 300, 2),
+    (1, 17920, 1024, 300, 2), (2, 17920, 1024, 300, 1)])
 def test_gemm_wide(wide_eng, mode, Nout, K, R, terms):
     """CTA-pair GEMM against a 64-bit matmul of the same bf16 terms: the bounds of the 128-row kernel's tests, sums in fp32
     (1e-4 of the largest result), act one bf16 rounding of it (eight significant bits: half a unit in the last place is at
@@ -640,6 +641,36 @@ def test_prefill_passes_of_many_rows(harness, n_img, n_txt):
     run = harness.ParityRun(synth.CONFIGS["tiny"].replace(n_img=n_img, n_txt=n_txt))
     run.check_state()
     run.check_head_state()
+
+
+@pytest.mark.parametrize("prior,count", [(0, 700), (333, 701), (900, 740)])
+def test_prefill_in_one_call_equals_short_calls(harness, prior, count):
+    """A prefill whose query tiles fill the GPU (causal, 4 heads x 39 tiles and more, d 128: no key splits, up to 13 tiles of
+    128 keys to a CTA) against the same rows in calls of 50 (eight splits).  K/V rows are rounded alike and sums are added in
+    another order, so a bf16 result falls on the neighbouring value here and there: in the 2-norm no more than one rounding
+    of every value (2^-8 / sqrt(3) = 2.3e-3), and at most one unit in the last place (2^-7) of the largest.  The projections
+    are scaled so that the attention's output is as large as the residual."""
+    from paper_2609_00355_b200.binding import Engine
+    cfg = synth.CONFIGS["7b"].replace(n_layers=2, hidden=128, ffn=64, vocab=256, tree_N=16, block_B=4, topk=2)
+    tw, hw = synth.make_weights(cfg, "cuda")
+    for lw in tw["layers"]:
+        lw["wqkv"] *= 8
+    x = torch.randn(prior + count, cfg.hidden, generator=torch.Generator(device="cuda").manual_seed(9), device="cuda").to(torch.bfloat16)
+
+    def run(lengths):
+        eng = Engine(cfg, tw, hw, max_len=prior + count + 64)
+        at = 0
+        for n in [50] * (prior // 50) + [prior % 50] * (prior % 50 > 0) + lengths:
+            eng.glance_prefill(0, embeds=x[at:at + n].contiguous())
+            at += n
+        eng.check_device_status()
+        assert at == prior + count == int(eng.seq_len[0])
+        rows = [eng.gather_kv(0, 1, at), eng.gather_head_kv(0, at)]
+        return torch.stack([torch.cat([k, v], dim=-1)[prior:] for k, v in rows]).float()
+
+    one, short = run([count]), run([50] * (count // 50) + [count % 50] * (count % 50 > 0))
+    assert float((one - short).norm() / short.norm()) <= 2.3e-3
+    assert float((one - short).abs().amax()) <= 2 ** -7 * float(short.abs().amax())
 
 
 @pytest.mark.parametrize("first,count,status", [(0, 512, 0), (0, 513, -3), (3, 504, 0), (3, 505, -3)])
