@@ -23,8 +23,8 @@
 // never touched between tiles.  Loops over columns are kept rolled where they can be: every launch finds its
 // instructions cold, and a CTA of a short context runs this code two or three times.
 // Measured per layer at the 7B widths against 64-key tiles with two threads a row and two S/P buffers a group, us: 128 rows
-// over 8704 positions 72 -> 49, 8 x 64 rows over 1024..4096 97 -> 71, 1280 rows of a prefill 97 -> 42, 64 rows over 1536
-// 17.8 -> 16.2, one row 15 -> 13.3.  What is left of a long loop is the softmax warps (about 1.9 us per 128-key tile for
+// over 8704 positions 72 -> 46, 8 x 64 rows over 1024..4096 97 -> 71, 1280 rows of a prefill 97 -> 42, 64 rows over 1536
+// 17.8 -> 16.2, one row 15 -> 13.3.  What is left of a long loop is the softmax warps (1.85 us per 128-key tile for
 // 1.05 of MMAs), of a short one the start and the merge.
 // Warp roles: warp 0 = TMA producer, warp 1 = TMEM allocator + MMA issuer, warps 2..9 = softmax / epilogue.
 // The key splits of a tile form a thread-block cluster and are merged through distributed shared memory
@@ -734,10 +734,11 @@ int attention_tc_q_tiles(int T, int G) { return (T * G + QT - 1) / QT; }
 
 // Key splits per (sequence, kv head, q tile): the splits of a tile form a cluster, and all clusters of the
 // launch should be resident at once (a second wave would double the kernel's latency).  A launch that cannot fit
-// one wave split (several sequences) gets two splits: that halves the longest sequence's loop, which sets the
-// launch's duration, while larger clusters lose more than they gain once clusters queue for SMs (a cluster starts
+// one wave split (several sequences), but fits unsplit, gets two splits: that halves the longest sequence's loop, which sets
+// the launch's duration, while larger clusters lose more than they gain once clusters queue for SMs (a cluster starts
 // only when enough SMs of one GPC are free together: with 64-key tiles 8 sequences of 1024-4096 positions took 100 / 84 /
 // 102 / 154 us per layer with 1 / 2 / 4 / 8 splits; with 128-key tiles two splits take 70).
+// Beyond one CTA per SM unsplit (a long prefill, many sequences) there is nothing to fill, and it stays unsplit.
 int attention_tc_splits(int T, int G, int Hkv, int batch, int d) {
     const int base = attention_tc_q_tiles(T, G) * Hkv * batch;
     for (int s = MAX_SPLITS; s > 1; --s) {

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
     const int stage_bytes = BM * 128 + NB * 128;
     const int stages = a.stages;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // grid = (weight tiles, K splits, 128-row blocks) -- or, with more than one row block, (row blocks, K splits,
+    // grid = (weight tiles, K splits, row blocks of NP) -- or, with more than one row block, (row blocks, K splits,
     // weight tiles): CTAs are dispatched x-fastest, so the CTAs that stream the same weight tile for different row
     // blocks then start together and all but the first find the tile in L2 instead of reading HBM again
     const int tile_idx = a.rows_fastest ? blockIdx.z : blockIdx.x;
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(NTHR, (MODE == 0 || MODE == 2 || MODE == 5) ? 
     // processing (residual, rotary table, K/V row) are fetched ahead: those of a warp's first rows before the merge, under
     // which they travel.  Mode 3 then takes four rows at a time, one L2 latency for all of them (O at 577 rows, 8 rows a warp:
     // 19.7 -> 15.4 us); mode 4, whose body written out four times is slower than what it saves (every launch finds its
-    // instructions cold: QKV at 512 rows 28.9 -> 31.5 us), stays rolled and fetches a row's operands one row ahead.
+    // instructions cold: QKV at 512 rows 28.9 -> 31.5 us), stays rolled and fetches a row's operands two rows ahead.
     const int ew = warp - 2;                             // epilogue warp 0..7
     const int row_lo = (int)rank * RP;                   // first owned row (tile-local)
     const int my_rows = max(0, min(min(RP, NP - row_lo), a.R - r0 - row_lo));

@@ -5,9 +5,10 @@
 // a plug-in running inside a host framework's callback where allocation calls are off limits, or a
 // latency-critical loop that cannot tolerate the implicit device-wide synchronisation an allocation may
 // cause.  The regular path asks such callers for a workspace sized by glance_workspace_bytes(); this
-// entry point needs none.  Rows of up to 192 spans of 1024 entries are merged in the shared memory of a thread-block cluster;
-// for longer ones the two-stage top-k keeps its per-warp candidates and partial log-sum-exp terms in the file-scope array
-// below, which every GPU that loads the library holds until the process exits.  Its size bounds every request.
+// entry point needs none.  A few rows of up to 192 spans of 1024 entries are merged in the shared memory of a thread-block
+// cluster each; for longer or more rows the two-stage top-k keeps its per-warp candidates and partial log-sum-exp terms in the
+// file-scope array below, which every GPU that loads the library holds until the process exits.  What it holds is the stated
+// limit of a request, whichever way it goes.
 #include <mutex>
 
 #include "kernels.cuh"
